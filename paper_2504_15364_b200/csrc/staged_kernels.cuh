@@ -3,6 +3,7 @@
 // shared memory; the fused cluster kernel is preferred when a unit's keys fit a cluster.
 #pragma once
 #include "common.cuh"
+#include "segments.h"
 #include "select.cuh"
 
 namespace kd {
@@ -11,7 +12,6 @@ constexpr int kStagedThreads = 256;          // anchor / score kernels: 32 row g
 constexpr int kGroupsStaged = kStagedThreads / kLanesPerRow;
 constexpr int kSelectThreads = 1024;
 constexpr int kCompactThreads = 512;
-constexpr int kCompactRows = 128;            // rows staged per iteration (32 KB)
 
 // Row i of the logical concatenation [K_cache || k_block] of unit u (Eq. block_processing).
 __device__ __forceinline__ const uint4* concat_row(const uint4* cache, const uint4* block,

@@ -71,8 +71,6 @@ __device__ __forceinline__ double wide_sum_of_terms(int rows, const RowAt& row_a
 }
 
 // grid = U.  Also clears wide_move's counter and flags (2 * kMaxSegments per unit).
-constexpr int kMaxSegments = 8;    // wide_move: blocks per unit and tensor, at most
-constexpr int kHaloRows = 144;     // ... rows of a segment that are read ahead, at most (36 KB)
 __global__ void __launch_bounds__(kWideThreads)
 wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int raw_anchor,
                    double* __restrict__ anchor_sum, double* __restrict__ deltas, int ndeltas, float* __restrict__ mu,
@@ -227,11 +225,11 @@ wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ 
 // 16 x 8600 below 60; the gather of 16 x 20100 rows was most of the 405 us that a step took, now 124).
 // A segment owns a range [d0, d1) of destinations.  Rows move to lower places only, by at most m = (source of row d1 - 1) - (d1 -
 // 1), so the sources of its first d1 - m - d0 rows lie under d1, and nobody but itself writes there.  The last m rows may come
-// from where the next segment writes: the segment reads them into shared memory first and says so (flag, release); the next
-// one waits for that flag before its first store.  Segments are claimed from a counter in ascending order, so a block waits
-// only for one that is already running, and that one waits for nothing before it sets its flag.  The host picks several
-// segments only when at most kHaloRows rows are evicted per unit (then m <= kHaloRows).  Waits are bounded: one that runs out sets
-// the status word, and the block stores nothing.
+// from where the next segment writes, and not from further on (segments.h: m <= kHaloRows <= kMinSegmentRows): the segment
+// reads them into shared memory first and says so (flag, release); the next one waits for that flag before its first store.
+// Segments are claimed from a counter in ascending order, so a block waits only for one that is already running, and that one
+// waits for nothing before it sets its flag.  The host picks several segments only when at most kHaloRows rows are evicted per
+// unit.  Waits are bounded: one that runs out sets the status word, and the block stores nothing.
 __global__ void __launch_bounds__(kCompactThreads)
 wide_move_kernel(uint4* k_cache, uint4* v_cache, const uint4* __restrict__ new_k, const uint4* __restrict__ new_v,
                  int len, int B, int N, int segments, const int32_t* __restrict__ kept_idx, const int32_t* __restrict__ first_evicted,
@@ -251,9 +249,9 @@ wide_move_kernel(uint4* k_cache, uint4* v_cache, const uint4* __restrict__ new_k
     unsigned* flag = move_sync + 1 + (u * 2 + tensor) * kMaxSegments;
     // cache rows in front of the first evicted row stay; block rows (index >= len) always move
     const int first = min(first_evicted[u], len);
-    const int per = ((N - first + segments - 1) / segments + kCompactRows - 1) / kCompactRows * kCompactRows;
-    const int d0 = min(N, first + s * per), d1 = min(N, d0 + per);
-    const int m = d1 > d0 && d1 < N ? min(src_of[d1 - 1] - (d1 - 1), d1 - d0) : 0;   // (the last segment has no successor)
+    const Segment seg = segment_of(first, N, segments, s);
+    const int d0 = seg.d0, d1 = seg.d1;
+    const int m = rows_read_ahead(seg, N, d1 > d0 ? src_of[d1 - 1] : 0);
     auto load_row = [&](int d, int c) {
         const int src = src_of[d];
         return KD_ROW_OK(src, len + B, status) ? concat_row(cache, block, u, src, len, B, N)[c] : make_uint4(0, 0, 0, 0);

@@ -61,6 +61,27 @@ def test_units_moved_by_several_blocks(U, N, B, length):
     kd.close()
 
 
+@pytest.mark.parametrize("U,N,at", [(16, 9000, 8000), (16, 9000, 8850), (3, 4111, 3300)])
+def test_a_run_of_evicted_rows_near_the_end_moved_by_several_blocks(U, N, at):
+    # as many rows go as a block reads ahead, and all behind them move by that much: eight short segments, whose sources lie as far
+    # on as their direct successor's
+    B = 144
+    g = torch.Generator().manual_seed(N + at)
+    k, v, nk, nv = (torch.randn(U, rows, 128, generator=g).to(torch.bfloat16) for rows in (N, N, B, B))
+    run = torch.randn(U, 1, 128, generator=g) + 0.02 * torch.randn(U, B, 128, generator=g)   # one direction: the largest cosines
+    k[:, at:at + B] = run.to(torch.bfloat16)
+    k, v, nk, nv = k.cuda(), v.cuda(), nk.cuda(), nv.cuda()
+    with pytest.MonkeyPatch.context() as m:
+        if N < 9000:
+            m.setenv("KEYDIFF_CLUSTER_SIZE", "1")
+        kd = KeyDiff(1, 1, U, 128, N, B)
+    assert kd.launch_info()["path"] == binding.KEYDIFF_PATH_STAGED
+    kd.set_len(N)
+    check(kd, k, v, nk, nv, N, N)
+    assert torch.equal(kd.scratch()["first_evicted"].cpu(), torch.full((U,), at, dtype=torch.int32))
+    kd.close()
+
+
 def test_equal_scores_keep_the_older_token(monkeypatch):
     monkeypatch.setenv("KEYDIFF_CLUSTER_SIZE", "1")
     U, N, B = 2, 2500, 300
