@@ -2,30 +2,25 @@
 // the table and the ranking of a short list are enough.
 #pragma once
 #include "fused_kernel.cuh"   // kBins
+#include "sel_barrier.cuh"
 
 namespace kd {
 
-constexpr int kSelWarps = 8, kSelThreads = 32 * kSelWarps;
 constexpr int kSelList = 1024;    // keys under the first bound that are listed
 constexpr int kSelTies = 256;     // keys of the threshold bin ranked exactly
 constexpr int kSelDirect = 128;   // units of so few keys are ranked whole (at 230 keys that takes 143 instead of 124 us a step on 4000 units)
 constexpr int kMinBins = 1024;    // histogram of the classes' smallest keys
 
-__device__ __forceinline__ void sel_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kSelThreads) : "memory"); }
-
-// Number of selector threads with `p` (a barrier, too).
-__device__ __forceinline__ int sel_count(bool p) {
-    int r;
-    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %1, 0;\n\tbarrier.cta.red.popc.u32 %0, 1, %2, q;\n\t}" : "=r"(r) : "r"(static_cast<uint32_t>(p)), "n"(kSelThreads) : "memory");
-    return r;
-}
-
 struct SelectorScratch {   // 128-byte aligned
     int hist[kBins], min_hist[kMinBins];
     uint32_t list_key[kSelList]; int list_idx[kSelList];
     uint32_t tie_key[kSelTies]; int tie_idx[kSelTies];
-    int wtot[48];   // warp totals, warp minima and bounds
+    int wtot[48];   // 0 .. 7 warp totals, 16 .. 31 warp minima and bounds
     int misc[8];    // 0 listed keys, 1 the caller's, 2 / 3 broadcast, 6 keys of the threshold bin
+    // What lies between a word's last read and its next write.  misc[0]: written once per selection.  misc[2] / [3]: read behind the last
+    // barrier of a radix round, written behind the first ones of the next.  misc[6]: read behind the barrier in front of the ranking, reset
+    // behind the first barrier of select_evicted_any.  wtot[0 .. 7]: a scan begins with a barrier; between two crossings lies the pass
+    // that marks or lists.  wtot[16 .. 31]: written once per selection.
 };
 struct Selector {
     int* hist; int* min_hist; uint32_t* list_key; int* list_idx; uint32_t* tie_key; int* tie_idx;
@@ -148,6 +143,7 @@ __device__ __forceinline__ bool mark_smallest(const Visit& visit, uint32_t lo, u
 // 8-bit digits, then the newest of its equals.
 __device__ __noinline__ void select_evicted_any(const uint32_t* keys, int n, int E, uint32_t lo, uint32_t hi, int st, const Selector& s) {
     const int lane = st & 31, nwords = (n + 31) >> 5;
+    sel_sync();   // every warp has read misc[6], and with it that the list is crowded, before it is reset
     for (int b = st; b < kBins; b += kSelThreads) s.hist[b] = 0;
     for (int q = st; q < nwords; q += kSelThreads) s.bitmap[q] = 0;
     if (st == 0) s.misc[6] = 0;

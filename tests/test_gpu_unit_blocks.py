@@ -75,6 +75,37 @@ def test_equal_scores_keep_the_older_token(slots, N, B):
         caches=(cut(allk, 0, N), cut(allv, 0, N)))
 
 
+@pytest.mark.parametrize("entry", ["ordered", "slots", "staged"])
+@pytest.mark.parametrize("N,same,B", [(560, 300, 40), (700, 400, 40), (960, 900, 40), (640, 640, 300)])
+def test_one_direction_repeated_crowds_the_list(entry, N, same, B):
+    # more equal keys under the threshold than the selection's threshold bin may list, but not more than its list: the route that
+    # passes from the list to the whole table
+    U = 80
+    g = torch.Generator().manual_seed(N)
+    allk, allv = (torch.randn(U, N + 2 * B, 128, generator=g) for _ in range(2))
+    allk[:, torch.randperm(N, generator=g)[:same]] = torch.randn(U, 1, 128, generator=g)
+    allk, allv = allk.to(torch.bfloat16).cuda(), allv.to(torch.bfloat16).cuda()
+    cut = lambda t, a, b: t[:, a:b].contiguous()
+    blocks = [(cut(allk, N + s * B, N + (s + 1) * B), cut(allv, N + s * B, N + (s + 1) * B)) for s in range(2)]
+    if entry != "staged":
+        run(U, N, B, N, entry == "slots", blocks=blocks, caches=(cut(allk, 0, N), cut(allv, 0, N)))
+        return
+    k, v = cut(allk, 0, N), cut(allv, 0, N)
+    static_k, static_v = k.clone(), v.clone()
+    kd = KeyDiff(1, 1, U, 128, N, B, path=binding.KEYDIFF_PATH_STAGED)
+    kd.set_len(N)
+    for nk, nv in blocks:
+        pre_k, pre_v = bits(k), bits(v)
+        kd.evict(k, v, nk, nv)
+        assert binding.evict_static(static_k, static_v, nk, nv, N) == N
+        torch.cuda.synchronize()
+        sc = kd.scratch()
+        compare.check_step(pre_k, pre_v, N, bits(nk), bits(nv), N, bits(k), bits(v), sc["scores"].cpu().numpy(), sc["kept_idx"].cpu().numpy(),
+                           n_threads=8)
+        assert torch.equal(k, static_k) and torch.equal(v, static_v)
+    kd.close()
+
+
 def test_two_contexts_on_two_streams_do_not_disturb_each_other():
     wl = synth.Workload("t", 1, 1, 200, 128, 400, 40, "outlier", 400 + 10 * 40, 84)
     out = []
