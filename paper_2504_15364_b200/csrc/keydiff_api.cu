@@ -189,11 +189,18 @@ FusedKernel fused_instance(int reg_rows, int* built, bool one_pass = false, bool
     return few_pre ? fused_instance_of<true, 1>(reg_rows, built) : fused_instance_of<true, 4>(reg_rows, built);
 }
 
+// Lets a kernel be launched with up to kSmemLimit bytes of dynamic shared memory.  The limit belongs to the kernel on the device, not to a
+// context: it is always the same, so that a context created later for smaller units does not lower it under an earlier one.
+template <typename Kernel>
+bool allow_shared_memory(Kernel kern, int bytes = kd::kSmemLimit) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+}
+
 // Co-resident clusters of `C` CTAs of the kernel `kern` with `smem` bytes each.
 template <typename Kernel>
 int max_active_clusters(Kernel kern, int C, int smem, int sm_count) {
     using namespace kd;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return 0;
+    if (!allow_shared_memory(kern)) return 0;
     if (C > 8 && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(C * sm_count);
@@ -243,7 +250,7 @@ bool plan_fused(keydiff_ctx* c, int sm_count) {
         }
     }
     if (!found) return false;
-    // the attributes of the chosen instance (the loop may have left another size's values behind)
+    // the attributes of the three kernels of the chosen instance (the loop has set those of the two-pass kernel alone)
     int built = 0;
     return max_active_clusters(fused_instance(c->fused_reg_rows, &built, false), c->cluster, c->fused_smem_bytes, sm_count) >= 1 &&
            max_active_clusters(fused_instance(c->fused_reg_rows, &built, true, false), c->cluster, c->fused_smem_bytes, sm_count) >= 1 &&
@@ -383,7 +390,7 @@ bool plan_unit(keydiff_ctx* c) {
     c->cluster = 1;
     c->unit_depth = depth;
     c->fused_smem_bytes = smem;
-    return cudaFuncSetAttribute(unit_instance(c), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+    return allow_shared_memory(unit_instance(c));
 }
 
 int launch_unit(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int B, cudaStream_t st) {
@@ -546,7 +553,7 @@ int launch_staged(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const u
 bool alloc_wide(keydiff_ctx* c) {
     return kd_malloc(&c->mu, sizeof(float) * c->U * kd::kMuStride) == cudaSuccess &&
            kd_malloc(&c->move_sync, sizeof(unsigned) * (1 + c->U * 2 * kd::kMaxSegments)) == cudaSuccess &&
-           cudaFuncSetAttribute(kd::wide_move_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMoveSmem) == cudaSuccess;
+           allow_shared_memory(kd::wide_move_kernel, kMoveSmem);
 }
 
 int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
@@ -609,16 +616,12 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
              cudaMemset(c->moved_rows, 0, sizeof(unsigned long long)) == cudaSuccess;
     }
     if (ok) {
-        ok = cudaFuncSetAttribute(kd::select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kMaxSelectSmem) == cudaSuccess &&
-             cudaFuncSetAttribute(kd::wide_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  kWideSelectSmem) == cudaSuccess;
+        ok = allow_shared_memory(kd::select_kernel, kMaxSelectSmem) && allow_shared_memory(kd::wide_select_kernel, kWideSelectSmem);
     }
     if (ok && cfg->compaction == KEYDIFF_COMPACT_SLOT_REUSE) {
         ok = kd_malloc(&c->pos, sizeof(int32_t) * U * cfg->budget) == cudaSuccess &&
              cudaMemset(c->pos, 0, sizeof(int32_t) * U * cfg->budget) == cudaSuccess &&
-             cudaFuncSetAttribute(kd::slot_place_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  std::max(48 * 1024, 8 * cfg->max_block)) == cudaSuccess;
+             allow_shared_memory(kd::slot_place_kernel, kMaxSelectSmem);   // (8 bytes per row of a block: checked above)
     }
     if (ok) ok = cudaDeviceSynchronize() == cudaSuccess;
     if (ok && cfg->path != KEYDIFF_PATH_STAGED) {

@@ -66,6 +66,32 @@ def test_allocation_failure_in_create_releases_everything(compaction):
     kd.close()
 
 
+@pytest.mark.parametrize("slots,path,U,big,small", [
+    (False, 2, 8, (2048, 128), (1024, 128)), (True, 2, 8, (4096, 128), (1024, 128)),       # one cluster per unit
+    (False, 0, 90, (800, 150), (100, 20)), (True, 0, 8, (500, 100), (60, 40)), (True, 0, 150, (2040, 130), (1500, 100)),   # one block
+    (True, 1, 2, (9000, 8000), (200, 64))])                                                # four launches, placement of 8000 rows
+def test_a_context_for_smaller_units_leaves_the_larger_one_working(slots, path, U, big, small):
+    # the limit on a kernel's dynamic shared memory is the device's, not the context's
+    kds = [KeyDiff(1, 1, U, 128, N, B, path=path, compaction=int(slots)) for N, B in (big, small)]
+    for kd, (N, B) in zip(kds, (big, small)):
+        wl = synth.Workload("t", 1, 1, U, 128, N, B, "outlier", N + 2 * B, 41)
+        k, v, stream = synth.prefilled_cache(wl, DEV)
+        kd.set_len(N)
+        for step in range(2):
+            nk, nv = stream.next_block(B)
+            pre_k, pre_v = bits(k), bits(v)
+            kd.evict(k, v, nk, nv)
+            torch.cuda.synchronize()
+            sc = kd.scratch()
+            if step == 0 and not slots:
+                compare.check_step(pre_k, pre_v, N, bits(nk), bits(nv), N, bits(k), bits(v), sc["scores"].cpu().numpy(), sc["kept_idx"].cpu().numpy(),
+                                   n_threads=8)
+            elif step == 0:
+                compare.check_step_slots(pre_k, pre_v, np.tile(np.arange(N), (U, 1)), N, N, bits(nk), bits(nv), N, bits(k), bits(v),
+                                         sc["scores"].cpu().numpy(), sc["kept_idx"].cpu().numpy(), kd.positions()[0].cpu().numpy(), n_threads=8)
+        kd.close()
+
+
 def run_slot_stream(wl, window, steps, incremental, resume_at=None):
     """Slot-reuse stream of `steps` evicting steps; with resume_at = s the caches, positions and next position
     are saved after step s, the ctx is destroyed, and a NEW ctx continues from the saved state."""
