@@ -16,10 +16,10 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", 
               "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]
 
 
-def _stale() -> bool:
-    if not LIB.exists():
+def _stale(lib: Path) -> bool:
+    if not lib.exists():
         return True
-    t = LIB.stat().st_mtime
+    t = lib.stat().st_mtime
     deps = list(CSRC.glob("*.cu")) + list(CSRC.glob("*.cuh")) + list(CSRC.glob("*.h")) + list((PKG.parent / "include").glob("*.h"))
     return any(p.stat().st_mtime > t for p in deps)
 
@@ -48,7 +48,7 @@ def build_library(force: bool = False, verbose: bool = False, phase_stamps: bool
     debug_checks=True the variant libkeydiff_debug.so (-DKEYDIFF_DEBUG_CHECKS: row indices are range-checked)."""
     build_pycall(force)
     out = STAMPS_LIB if phase_stamps else DEBUG_LIB if debug_checks else LIB
-    if not force and not phase_stamps and not debug_checks and not _stale():
+    if not force and not _stale(out):
         return out
     nvcc = os.environ.get("NVCC", "nvcc")
     tmp = out.with_suffix(f".{os.getpid()}.tmp")

@@ -648,7 +648,10 @@ __device__ __noinline__ void full_select_plan(const uint32_t* keys, int n, int N
 // row that enters the cache adds exactly what it takes away when it is evicted, and no fp32 partial sum of the
 // size of the anchor appears anywhere (an anchor over keys that point in many directions is a cancelling sum;
 // fp32 partial sums would limit it, and with it every score, to about 1e-7 / ||mu||).
-// warp_row_terms (below) forms these terms; both fused kernels and the staged kernels use the same products.
+// warp_row_terms (below) forms these terms, and block_sum_of_terms (row_terms.cuh) the same bits; whatever adds block rows or takes
+// evicted rows out uses one of the two.  A sum rebuilt from all rows starts with a fixed error instead: except in the block
+// per unit, four to six rows are added in fp32 before they enter the double sum (the anchor of thousands of rows is off by less
+// than one row's rounding), and since the rows leave by their terms, that error stays as it is until the next rebuild.
 
 // Evicted tokens before each word of the bitmap: wlocal[w] = number of set bits in words [0, w).  All threads
 // call; uses sel.warp_gt, sel.hist[32..48) and misc[5], misc[6]; ends with a CTA barrier.

@@ -7,6 +7,7 @@
 #include <cstdlib>
 #include <mutex>
 #include <new>
+#include <vector>
 
 #include "common.cuh"
 #include "staged_kernels.cuh"
@@ -895,6 +896,22 @@ int keydiff_selftest_bounded_wait(int32_t* status_device, int32_t polls, void* s
     KD_CUDA(cudaGetLastError());
     return KEYDIFF_OK;
 }
+
+#ifdef KEYDIFF_DEBUG_CHECKS
+// Debug-checks build only: the running sum of the cached rows' anchor terms as the latest step left it, [U][128] doubles, to out_host.
+// KEYDIFF_ERR_STATE when the next step would rebuild it.  Synchronises the device.
+__attribute__((visibility("default"))) int keydiff_debug_anchor_sum(const keydiff_ctx* ctx, double* out_host) {
+    if (!ctx || !out_host) return KEYDIFF_ERR_INVALID_ARG;
+    if (!ctx->anchor_valid) return KEYDIFF_ERR_STATE;
+    const size_t units = ctx->U, ranks = ctx->anchor_delta ? ctx->cluster : 0;
+    std::vector<double> deltas(units * ranks * kd::kHeadDim);
+    KD_CUDA(cudaDeviceSynchronize());
+    KD_CUDA(cudaMemcpy(out_host, ctx->anchor_sum[ctx->anchor_par], sizeof(double) * units * kd::kHeadDim, cudaMemcpyDeviceToHost));
+    if (ranks > 0) KD_CUDA(cudaMemcpy(deltas.data(), ctx->anchor_delta, sizeof(double) * deltas.size(), cudaMemcpyDeviceToHost));
+    for (size_t i = 0; i < deltas.size(); ++i) out_host[i / kd::kHeadDim / ranks * kd::kHeadDim + i % kd::kHeadDim] += deltas[i];
+    return KEYDIFF_OK;
+}
+#endif
 
 #ifdef KEYDIFF_PHASE_STAMPS
 // Phase-stamp build only: copies the per-CTA, per-phase nanosecond totals of the fused kernel to out_host

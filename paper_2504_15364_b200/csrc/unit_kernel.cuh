@@ -9,6 +9,7 @@
 // Long units: HBM, at 85-88 % of its copy rate with slot reuse (512 x 8224 rows: 197 us, 172 at the full rate).
 #pragma once
 #include "low_select.cuh"
+#include "row_terms.cuh"
 #include "slot_kernel.cuh"      // issue_rows
 #include "staged_kernels.cuh"   // concat_row
 
@@ -53,63 +54,6 @@ struct UnitParams {
     int32_t* kept_mirror;
 };
 
-// Sum of the anchor terms of `rows` rows over the block, row r at row_at(r): channel st's total in threads st < 128.  The
-// terms are those of warp_row_terms, bit for bit: lane j of a half warp holds channels 4j .. 4j+3 and 64+4j .. 64+4j+3, so
-// its sum of the two four-term chains is what the butterfly's first exchange would give; the rest of the butterfly
-// follows.  Two rows per warp and step, eight requested together.  A row that is not there counts as zeros, which add
-// nothing.  table: [8][128] doubles; one barrier inside, behind which every row has been read.
-template <typename RowAt>
-__device__ __forceinline__ double unit_sum_of_terms(int rows, const RowAt& row_at, float inv_eps, bool raw, double* table, int st) {
-    constexpr int kDeep = 4;
-    const int wid = st >> 5, lane = st & 31, half = lane >> 4, j = lane & 15;
-    double acc[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-#pragma unroll 1
-    for (int r0 = 2 * wid + half; r0 - half < rows; r0 += 2 * kUnitWarps * kDeep) {
-        uint2 a[kDeep], b[kDeep];
-#pragma unroll
-        for (int k = 0; k < kDeep; ++k) {
-            const int r = r0 + 2 * kUnitWarps * k;
-            a[k] = make_uint2(0, 0); b[k] = a[k];
-            if (r < rows) { const uint2* row = reinterpret_cast<const uint2*>(row_at(r)); a[k] = row[j]; b[k] = row[j + 16]; }
-        }
-        float ss[kDeep];
-#pragma unroll
-        for (int k = 0; k < kDeep; ++k) {
-            const float x0 = bf16_lo(a[k].x), x1 = bf16_hi(a[k].x), x2 = bf16_lo(a[k].y), x3 = bf16_hi(a[k].y);
-            const float y0 = bf16_lo(b[k].x), y1 = bf16_hi(b[k].x), y2 = bf16_lo(b[k].y), y3 = bf16_hi(b[k].y);
-            ss[k] = fmaf(x3, x3, fmaf(x2, x2, fmaf(x1, x1, x0 * x0))) + fmaf(y3, y3, fmaf(y2, y2, fmaf(y1, y1, y0 * y0)));
-        }
-#pragma unroll
-        for (int o = 8; o > 0; o >>= 1)
-#pragma unroll
-            for (int k = 0; k < kDeep; ++k) ss[k] += __shfl_xor_sync(0xffffffffu, ss[k], o);
-#pragma unroll
-        for (int k = 0; k < kDeep; ++k) {
-            const float inv = raw ? 1.0f : fminf(approx_rsqrt(ss[k]), inv_eps);
-            acc[0] += static_cast<double>(__fmul_rn(bf16_lo(a[k].x), inv)); acc[1] += static_cast<double>(__fmul_rn(bf16_hi(a[k].x), inv));
-            acc[2] += static_cast<double>(__fmul_rn(bf16_lo(a[k].y), inv)); acc[3] += static_cast<double>(__fmul_rn(bf16_hi(a[k].y), inv));
-            acc[4] += static_cast<double>(__fmul_rn(bf16_lo(b[k].x), inv)); acc[5] += static_cast<double>(__fmul_rn(bf16_hi(b[k].x), inv));
-            acc[6] += static_cast<double>(__fmul_rn(bf16_lo(b[k].y), inv)); acc[7] += static_cast<double>(__fmul_rn(bf16_hi(b[k].y), inv));
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], 16);
-    if (half == 0) {
-        double2* row = reinterpret_cast<double2*>(table + wid * kHeadDim + 4 * j);
-        row[0] = make_double2(acc[0], acc[1]); row[1] = make_double2(acc[2], acc[3]);
-        row[32] = make_double2(acc[4], acc[5]); row[33] = make_double2(acc[6], acc[7]);
-    }
-    __syncthreads();
-    double sum = 0.0;
-    if (st < kHeadDim) {
-#pragma unroll
-        for (int q = 0; q < kUnitWarps; ++q) sum += table[q * kHeadDim + st];
-    }
-    return sum;
-}
-
 template <bool kSlots, bool kRing>
 __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitParams p) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -146,7 +90,7 @@ __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitP
     {
         if (tid < kHeadDim && !p.rebuild) sum = p.anchor_sum[static_cast<size_t>(u) * kHeadDim + tid];
         const int first = p.rebuild ? 0 : len;
-        sum += unit_sum_of_terms(n - first, [&](int r) { return concat_row(p.k_cache, p.new_k, u, first + r, len, B, N); }, inv_eps, raw, sums, tid);
+        sum += block_sum_of_terms(n - first, [&](int r) { return concat_row(p.k_cache, p.new_k, u, first + r, len, B, N); }, inv_eps, raw, sums, tid);
         if (tid < kHeadDim) mu[tid] = static_cast<float>(sum / static_cast<double>(n));
         __syncthreads();
     }
@@ -239,7 +183,7 @@ __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitP
                 if (mirror) mirror[d] = i;
             }
         // (the barrier inside makes the list visible and lies behind every read of an evicted row)
-        const double gone = unit_sum_of_terms(E, [&](int r) { return concat_row(p.k_cache, p.new_k, u, min(max(ev_of[r], 0), n - 1), len, B, N); },
+        const double gone = block_sum_of_terms(E, [&](int r) { return concat_row(p.k_cache, p.new_k, u, min(max(ev_of[r], 0), n - 1), len, B, N); },
                                               inv_eps, raw, sums, tid);
         if (tid < kHeadDim) p.anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum - gone;
         const int first_moved = min(first_evicted, len);   // block rows always move into the cache
@@ -293,7 +237,7 @@ __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitP
             atomicAdd(p.moved_rows, static_cast<unsigned long long>(kb));
         }
         // (the barrier inside makes the lists visible and lies behind every read of an evicted row)
-        const double gone = unit_sum_of_terms(E, [&](int r) { return concat_row(p.k_cache, p.new_k, u, min(max(ev_of[r], 0), n - 1), len, B, N); },
+        const double gone = block_sum_of_terms(E, [&](int r) { return concat_row(p.k_cache, p.new_k, u, min(max(ev_of[r], 0), n - 1), len, B, N); },
                                               inv_eps, raw, sums, tid);
         if (tid < kHeadDim) p.anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum - gone;
 #pragma unroll 2

@@ -6,76 +6,32 @@
 //   wide_select   exact top-N, kept-index list; the evicted rows' terms leave the running sum
 //   compact_kernel (staged_kernels.cuh), or for few units wide_move, which gives a unit several blocks per tensor
 //
-// The running sum cannot drift: a row's terms are a fixed bit pattern, the fp32 products of its elements and its fp32
-// reciprocal norm (IEEE square root and division), added and subtracted in double.
+// The running sum cannot drift: a row's terms are the fixed bit pattern that the other kernels add and take out as well
+// (row_terms.cuh), added and subtracted in double.
 //
 // What bounds it: HBM.  256 units of 16512 keys, 5.4 GB of traffic a step: 902 us; before, in the staged kernels, 1280 us (anchor and
 // score pass 308 + 229, selection 66, compaction 684).  Now the score pass takes 172 us (6.3 TB/s), the selection 30, the
 // compaction 683 (6.3 TB/s).
 #pragma once
 #include "low_select.cuh"
+#include "row_terms.cuh"
 #include "staged_kernels.cuh"
 
 namespace kd {
 
 constexpr int kWideThreads = 256, kWideGroups = kWideThreads / kLanesPerRow;
 constexpr int kWideDeep = 4;             // rows a row group requests together
+constexpr int kWideTermsDeep = 8;        // 128 block rows or evicted rows requested together
 constexpr int kMuStride = kHeadDim + 4;  // a unit's anchor and its norm
 static_assert(kWideDeep == 4, "group_sum_of4");
 static_assert(kWideThreads == kSelThreads, "wide_select runs the selector's 256 threads");
-
-// Sum of the anchor terms of `rows` rows, row r at row_at(r), over the block: channel c's total in thread c < 128.
-// table: [8][128] doubles; a barrier in front of the return lies behind every read of a row.
-template <typename RowAt>
-__device__ __forceinline__ double wide_sum_of_terms(int rows, const RowAt& row_at, float eps, bool raw, double* table) {
-    const int tid = threadIdx.x, g = tid >> 3, t = tid & 7, lane = tid & 31;
-    double acc[16];
-#pragma unroll
-    for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-#pragma unroll 1
-    for (int r0 = 0; r0 < rows; r0 += kWideGroups * kWideDeep) {   // (the same trip count in every lane)
-        uint4 a[kWideDeep], b[kWideDeep];
-#pragma unroll
-        for (int k = 0; k < kWideDeep; ++k) {
-            const int r = r0 + k * kWideGroups + g;
-            a[k] = make_uint4(0, 0, 0, 0); b[k] = a[k];
-            if (r < rows) { const uint4* row = row_at(r); a[k] = row[t]; b[k] = row[t + 8]; }
-        }
-#pragma unroll
-        for (int k = 0; k < kWideDeep; ++k) {
-            float x[16];
-            unpack_row(a[k], b[k], x);
-            const float r = sqrtf(row_sumsq(x));
-            const float inv = raw ? 1.0f : 1.0f / fmaxf(r, eps);   // (a row that is not there is zero: its terms add nothing)
-#pragma unroll
-            for (int j = 0; j < 16; ++j) acc[j] += static_cast<double>(__fmul_rn(x[j], inv));
-        }
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 8);
-        acc[j] += __shfl_xor_sync(0xffffffffu, acc[j], 16);
-    }
-    if (lane < 8) {
-#pragma unroll
-        for (int j = 0; j < 16; j += 2)
-            *reinterpret_cast<double2*>(&table[(tid >> 5) * kHeadDim + lane_channel(t, j)]) = make_double2(acc[j], acc[j + 1]);
-    }
-    __syncthreads();
-    double sum = 0.0;
-    if (tid < kHeadDim) {
-#pragma unroll
-        for (int w = 0; w < kWideThreads / 32; ++w) sum += table[w * kHeadDim + tid];
-    }
-    return sum;
-}
 
 // grid = U.  Also clears wide_move's counter and flags (2 * kMaxSegments per unit).
 __global__ void __launch_bounds__(kWideThreads)
 wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int raw_anchor,
                    double* __restrict__ anchor_sum, double* __restrict__ deltas, int ndeltas, float* __restrict__ mu,
                    unsigned* __restrict__ move_sync) {
-    __shared__ double table[kWideThreads / 32 * kHeadDim];
+    __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     __shared__ float mu_sh[kHeadDim];
     grid_dependency_wait();
     const int u = blockIdx.x, tid = threadIdx.x;
@@ -93,7 +49,8 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
                 delta = 0.0;
             }
     }
-    const double sum = run + wide_sum_of_terms(B, [&](int r) { return blk + static_cast<size_t>(r) * kRowVec; }, eps, raw_anchor != 0, table);
+    const double sum = run + block_sum_of_terms<kWideTermsDeep>(B, [&](int r) { return blk + static_cast<size_t>(r) * kRowVec; }, 1.0f / eps,
+                                                                raw_anchor != 0, table, tid);
     if (tid < kHeadDim) {
         anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum;
         mu_sh[tid] = static_cast<float>(sum / static_cast<double>(n));
@@ -175,7 +132,7 @@ wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ 
                    int32_t* __restrict__ kept_idx, int32_t* __restrict__ first_evicted, unsigned long long* __restrict__ moved_rows) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(128) SelectorScratch scratch;
-    __shared__ double table[kSelWarps * kHeadDim];
+    __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     grid_dependency_wait();
     const int u = blockIdx.x, tid = threadIdx.x, n = len + B, E = n - N, nwords = (n + 31) >> 5;
     uint32_t* keys = reinterpret_cast<uint32_t*>(smem);
@@ -215,8 +172,8 @@ wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ 
         if (!(wd & bit)) out[i - before[i >> 5] - __popc(wd & (bit - 1u))] = i;
     }
     if (!anchor_sum) return;   // (the staged path keeps no sum)
-    const double sum = wide_sum_of_terms(E, [&](int r) { return concat_row(k_cache, new_k, u, static_cast<int>(gone[r]), len, B, N); },
-                                         eps, raw_anchor != 0, table);
+    const double sum = block_sum_of_terms<kWideTermsDeep>(E, [&](int r) { return concat_row(k_cache, new_k, u, static_cast<int>(gone[r]), len, B, N); },
+                                                          1.0f / eps, raw_anchor != 0, table, tid);
     if (tid < kHeadDim) anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] -= sum;
 }
 
