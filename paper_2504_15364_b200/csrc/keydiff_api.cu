@@ -164,11 +164,11 @@ cudaError_t launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cuda
 }
 
 cudaError_t launch_append(uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int len, int B, int N, int U,
-                          int32_t* pos, int next_pos, cudaStream_t st) {
+                          int32_t* pos, int next_pos, int pos_rows, cudaStream_t st) {
     using namespace kd;
     const int per_block = kAppendThreads * kAppendWords;
     return launch(append_kernel, dim3((B * kRowVec + per_block - 1) / per_block, U, 2), kAppendThreads, 0, st, 0, true,
-                  kc, vc, nk, nv, len, B, N, pos, next_pos);
+                  kc, vc, nk, nv, len, B, N, pos, next_pos, pos_rows);
 }
 
 using FusedKernel = void (*)(kd::FusedParams);
@@ -685,15 +685,17 @@ int keydiff_evict(keydiff_ctx* ctx, void* k_cache, void* v_cache, const void* ne
     if (slot_reuse(ctx)) {
         if (ctx->next_pos + block_B > 0x7fffffffLL) return KEYDIFF_ERR_STATE;   // positions are int32
         if (ctx->pos_stale && ctx->len > 0) {
-            // the cache as the caller declared it: slot s holds token s (an empty cache has no slot to describe)
+            // the cache as the caller declared it: slot s holds token s (for an empty cache the append writes it, and an
+            // evicting step fills every slot)
             const int total = ctx->U * N;
             KD_CUDA(launch(kd::pos_iota_kernel, dim3((total + 255) / 256), 256, 0, st, 0, true, ctx->pos, N, total));
         }
-        ctx->pos_stale = false;
     }
     if (n <= N) {
         // Sec. 2.3: the budget is not exceeded, nothing is evicted
-        KD_CUDA(launch_append(kc, vc, nk, nv, ctx->len, block_B, N, ctx->U, ctx->pos, static_cast<int>(ctx->next_pos), st));
+        KD_CUDA(launch_append(kc, vc, nk, nv, ctx->len, block_B, N, ctx->U, ctx->pos, static_cast<int>(ctx->next_pos),
+                              ctx->pos_stale && ctx->len == 0 ? N : block_B, st));
+        ctx->pos_stale = false;
         ctx->len = n;
         ctx->next_pos += block_B;
         ctx->anchor_valid = false;   // the appended rows are not in the running anchor
@@ -704,6 +706,7 @@ int keydiff_evict(keydiff_ctx* ctx, void* k_cache, void* v_cache, const void* ne
                      : ctx->wide || single              ? launch_wide(ctx, kc, vc, nk, nv, block_B, st)
                                                         : launch_staged(ctx, kc, vc, nk, nv, block_B, st);
     if (lrc != KEYDIFF_OK) return lrc;
+    ctx->pos_stale = false;
     ctx->len = N;
     ctx->next_pos += block_B;
     return KEYDIFF_OK;
@@ -1014,7 +1017,7 @@ extern "C" int keydiff_evict_static(void* k_cache, void* v_cache, const void* ne
         if (attr.type == cudaMemoryTypeDevice && attr.device != dev) return KEYDIFF_ERR_STATE;
     }
     if (n <= N) {   // budget not exceeded: plain append, no scratch involved
-        KD_CUDA(launch_append(kc, vc, nk, nv, len, block_B, N, U, nullptr, 0, st));
+        KD_CUDA(launch_append(kc, vc, nk, nv, len, block_B, N, U, nullptr, 0, 0, st));
         return KEYDIFF_OK;
     }
     if (n * 4 > kMaxSelectSmem) return KEYDIFF_ERR_TOO_LARGE;

@@ -299,13 +299,14 @@ __global__ void pos_iota_kernel(int32_t* __restrict__ pos, int N, int total) {
 }
 
 // Step a0 when the budget is not exceeded: rows [len, len+B) <- block rows, K and V; with slot reuse (pos != nullptr) slot
-// len + j then holds token next_pos + j.  Four 128-bit words per thread, requested together: with one word per thread the
+// len + j then holds token next_pos + j, for j < pos_rows: the block's rows, or all slots in the first step of a sequence, which
+// leaves the identity in the slots that are still empty.  Four 128-bit words per thread, requested together: with one word per thread the
 // launch of the blocks bounds the call.  grid = (ceil(B*16 / (4*threads)), U, 2).
 constexpr int kAppendThreads = 256, kAppendWords = 4;
 __global__ void __launch_bounds__(kAppendThreads)
 append_kernel(uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
               const uint4* __restrict__ new_k, const uint4* __restrict__ new_v,
-              int len, int B, int N, int32_t* __restrict__ pos, int next_pos) {
+              int len, int B, int N, int32_t* __restrict__ pos, int next_pos, int pos_rows) {
     grid_dependency_wait();
     const int u = blockIdx.y, total = B * kRowVec;
     uint4* cache = (blockIdx.z == 0 ? k_cache : v_cache) + (static_cast<size_t>(u) * N + len) * kRowVec;
@@ -318,7 +319,7 @@ append_kernel(uint4* __restrict__ k_cache, uint4* __restrict__ v_cache,
     for (int j = 0; j < kAppendWords; ++j) { const int q = q0 + j * kAppendThreads; if (q < total) cache[q] = w[j]; }
     grid_dependency_trigger();
     if (pos && blockIdx.z == 0)
-        for (int j = blockIdx.x * kAppendThreads + threadIdx.x; j < B; j += gridDim.x * kAppendThreads)
+        for (int j = blockIdx.x * kAppendThreads + threadIdx.x; j < pos_rows; j += gridDim.x * kAppendThreads)
             pos[static_cast<size_t>(u) * N + len + j] = next_pos + j;
 }
 

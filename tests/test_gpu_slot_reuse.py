@@ -301,3 +301,25 @@ def test_units_beyond_the_register_select(U, N, B, w):
     for step in range(2):
         checked_step(kd, k_cache, v_cache, *stream.next_block(B), 0, w, after_set_len=step == 0)
     kd.close()
+
+
+@pytest.mark.parametrize("N", [200, 1500])
+def test_the_first_step_of_a_sequence_writes_the_identity_into_all_slots(N):
+    # a second sequence on the same ctx: slots that it has not filled yet do not show positions of the first
+    wl = synth.Workload("t", 1, 1, 4, 128, N, 64, "outlier", 3 * N, 91)
+    stream = synth.KVStream(wl, "cuda")
+    k, v = (torch.zeros(4, N, 128, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    kd = KeyDiff(1, 1, 4, 128, N, 64, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
+    ident = torch.arange(N, dtype=torch.int32, device="cuda").expand(4, N)
+    for again in (kd.reset, lambda: kd.set_len(0)):
+        kd.evict(k, v, *stream.next_block(64))
+        assert torch.equal(kd.positions()[0], ident)
+        while kd.len < N:
+            kd.evict(k, v, *stream.next_block(64))
+        for _ in range(3):
+            kd.evict(k, v, *stream.next_block(64))
+        assert not torch.equal(kd.positions()[0], ident)
+        again()
+    kd.evict(k, v, *stream.next_block(1))
+    assert torch.equal(kd.positions()[0], ident) and kd.positions()[1] == 1
+    kd.close()
