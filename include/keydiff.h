@@ -113,7 +113,8 @@ typedef struct {
     int32_t max_block;     /* largest B ever passed to keydiff_evict (Sec. 2.4), >= 1 */
     int32_t dtype;         /* KEYDIFF_BF16 */
     int32_t path;          /* KEYDIFF_PATH_* */
-    float   eps;           /* eps of App. B.1's max(.,eps); 0 selects the default 1e-8 */
+    float   eps;           /* eps of App. B.1's max(.,eps); 0 selects the default 1e-8; a value below the
+                              smallest normal number (1.2e-38) counts as that number */
     int32_t device;        /* CUDA device ordinal */
     int32_t anchor_mode;   /* KEYDIFF_ANCHOR_*: which mean is the anchor (Sec. 3.2) */
     int32_t recent_window; /* w >= 0 most recent tokens that are never evicted (Sec. 3.2, "KeyDiff with
@@ -294,7 +295,7 @@ KEYDIFF_API int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, i
  * same in-place compaction in token order), but keeps no context: the caller passes the current
  * cache length `len` (0 <= len <= budget_N) and tracks the new one itself, min(budget_N, len +
  * block_B).  k_cache/v_cache: device, in/out, [n_units][budget_N][128] bf16; new_k/new_v: device,
- * read only, [n_units][block_B][128] bf16; all 16-byte aligned.  eps: 0 selects 1e-8.
+ * read only, [n_units][block_B][128] bf16; all 16-byte aligned.  eps: as in keydiff_config.
  * Asynchronous on `stream`.
  *
  * Limit: the step's scratch -- n_units * (8*(len+block_B) + 4*budget_N + 4) bytes plus the anchor

@@ -3,6 +3,7 @@
 #include "../../include/keydiff.h"
 
 #include <algorithm>
+#include <cfloat>
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
@@ -28,6 +29,10 @@ inline bool cuda_ok(cudaError_t e) {
 #define KD_CUDA(call) do { if (!cuda_ok(call)) return KEYDIFF_ERR_CUDA; } while (0)
 
 constexpr float kDefaultEps = 1e-8f;
+// The eps that the kernels get.  Not below the smallest normal number: 1/eps must be finite (a key of zeros, or a row that is not there and
+// counts as one, adds its zeros times min(1/||k||, 1/eps) to the anchor), and the kernels' products of norms are flushed to
+// zero below it anyway.
+inline float effective_eps(float eps) { return eps > 0.f ? std::max(eps, FLT_MIN) : kDefaultEps; }
 
 // Launch-tuning aids (named in include/keydiff.h): read from the environment ONCE, by keydiff_create; a step
 // never looks at the environment.  A value < 0 means "not set".
@@ -590,7 +595,7 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
     c->cfg = *cfg;
     c->U = static_cast<int>(U);
     c->nmax = static_cast<int>(nmax);
-    c->eps = cfg->eps > 0.f ? cfg->eps : kDefaultEps;
+    c->eps = effective_eps(cfg->eps);
     c->sm_count = prop.multiProcessorCount;
     c->tune_cluster = env_int("KEYDIFF_CLUSTER_SIZE");
     c->tune_stagger_ns = env_int("KEYDIFF_STAGGER_NS");
@@ -1041,7 +1046,7 @@ extern "C" int keydiff_evict_static(void* k_cache, void* v_cache, const void* ne
     // the array still holds the previous call's contents; the counter accumulates, so it is the
     // one part that must start from zero (everything else is fully overwritten before it is read)
     KD_CUDA(cudaMemsetAsync(moved, 0, sizeof(unsigned long long), st));
-    const float e = eps > 0.f ? eps : kDefaultEps;
+    const float e = effective_eps(eps);
     const int nn = static_cast<int>(n);
     const int rows_per_split = (nn + splits - 1) / splits;
     const dim3 grid(splits, U);

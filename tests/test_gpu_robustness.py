@@ -92,6 +92,29 @@ def test_a_context_for_smaller_units_leaves_the_larger_one_working(slots, path, 
         kd.close()
 
 
+@pytest.mark.parametrize("U,N,B,slots,path,cluster", [
+    (90, 240, 17, 0, 0, 0), (90, 240, 17, 1, 0, 0), (2, 1536, 100, 0, 2, 0), (8, 4000, 33, 1, 0, 0), (3, 1300, 17, 0, 0, 1), (3, 700, 17, 0, 1, 0)])
+def test_an_eps_whose_reciprocal_overflows_changes_nothing_for_ordinary_keys(monkeypatch, U, N, B, slots, path, cluster):
+    # the keys' norms are far above either eps, but for one key of zeros, whose terms are zeros and whose score is 0 under both
+    if cluster:
+        monkeypatch.setenv("KEYDIFF_CLUSTER_SIZE", str(cluster))
+    wl = synth.Workload("t", 1, 1, U, 128, N, B, "outlier", N + 4 * B, 43)
+    k0, v0, stream = synth.prefilled_cache(wl, DEV)
+    k0[:, 5] = 0
+    blocks = [stream.next_block(B) for _ in range(3)]
+    out = []
+    for eps in (0.0, 1e-39):
+        k, v = k0.clone(), v0.clone()
+        kd = KeyDiff(1, 1, U, 128, N, B, eps=eps, path=path, compaction=slots)
+        kd.set_len(N)
+        for nk, nv in blocks:
+            kd.evict(k, v, nk, nv)
+        out.append((k, v, kd.scratch()["kept_idx"].clone(), kd.scratch()["scores"].clone()))
+        kd.close()
+    assert not bool(out[1][3].isnan().any())
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
 def run_slot_stream(wl, window, steps, incremental, resume_at=None):
     """Slot-reuse stream of `steps` evicting steps; with resume_at = s the caches, positions and next position
     are saved after step s, the ctx is destroyed, and a NEW ctx continues from the saved state."""
