@@ -81,7 +81,6 @@ struct keydiff_ctx {
     int steps_since_full = 0;   // one-pass steps since the anchor was last recomputed from all rows
     double* anchor_sum[2] = {nullptr, nullptr};   // [U][128]
     double* anchor_delta = nullptr;               // [U][cluster][128]
-    bool delta_live = false;                      // the sum is anchor_sum[anchor_par] plus the deltas (the last step was the cluster kernel's)
     bool wide = false;                            // ordered layout, no cluster holds a unit: wide_kernels.cuh on anchor_sum[0]
     bool wide_single = false;                     // ordered layout, cluster kernel: steps that evict one row go to wide_kernels.cuh
     float* mu = nullptr;                          // [U][kMuStride], the running step's anchors
@@ -457,7 +456,7 @@ int launch_fused(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const ui
     KD_CUDA(launch(fused_instance(c->fused_reg_rows, &built, one_pass, few_pre), dim3(nclusters * c->cluster), kFusedThreads,
                    c->fused_smem_bytes, st, c->cluster, c->cluster == 1 || nclusters < c->fused_max_clusters, p));
     c->anchor_par ^= 1;
-    c->anchor_valid = c->delta_live = true;
+    c->anchor_valid = true;
     c->steps_since_full = one_pass ? c->steps_since_full + 1 : 0;
     return KEYDIFF_OK;
 }
@@ -495,7 +494,10 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     using namespace kd;
     const int N = c->cfg.budget, n = c->len + B, U = c->U;
     const int raw = c->cfg.anchor_mode == KEYDIFF_ANCHOR_RAW_MEAN;
+    // A step of single_evicted takes the sum from one buffer, and the deltas that the cluster kernel left beside it, and leaves it in the
+    // other, as that kernel does: steps captured in a graph go on from replay to replay whichever kernels serve them.
     double* sum = c->anchor_sum[c->anchor_par];
+    double* sum_out = c->wide_single ? c->anchor_sum[c->anchor_par ^ 1] : sum;
     if (!(c->incremental && c->anchor_valid && c->steps_since_full < 1024)) {   // (never a step of single_evicted)
         const int rows_per_split = (c->len + c->splits - 1) / c->splits;
         KD_CUDA(launch(anchor_partial_kernel, dim3(c->splits, U), kStagedThreads, 0, st, 0, true, kc, nk, c->len, 0, N, c->eps, rows_per_split,
@@ -506,9 +508,8 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     } else {
         ++c->steps_since_full;
     }
-    KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum,
-                   c->delta_live ? c->anchor_delta : nullptr, c->cluster, c->mu, c->move_sync));
-    c->delta_live = false;
+    KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum_out,
+                   c->anchor_delta, c->cluster, c->mu, c->move_sync));
     // parts of at least 256 rows, enough of them for several rounds of three blocks per SM
     const long long rows = 1LL * U * n;
     const int want = static_cast<int>(rows / (12LL * c->sm_count));
@@ -516,7 +517,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     KD_CUDA(launch(wide_score_kernel, dim3((n + rows_per_part - 1) / rows_per_part, U), kWideThreads, 0, st, 0, true, kc, nk, c->len, B, N,
                    c->eps, rows_per_part, c->nmax, c->mu, c->scores));
     KD_CUDA(launch(wide_select_kernel, dim3(U), kSelThreads, wide_select_smem(n), st, 0, true, kc, nk, c->scores, c->len, B, N, c->eps, raw,
-                   c->nmax, c->cfg.recent_window, sum, c->kept_idx, c->first_evicted, c->moved_rows));
+                   c->nmax, c->cfg.recent_window, sum_out, c->kept_idx, c->first_evicted, c->moved_rows));
     // as many blocks as run at once, three per SM, of at least 512 rows each (150 x 10600 rows: 408 us with 300 blocks, 474
     // with 600; 100 x 10600: 318 with 200, 287 with 400, 328 with 600); one per unit and tensor when the rows that a
     // block reads ahead do not fit its shared memory
@@ -527,6 +528,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     else
         KD_CUDA(launch(compact_kernel, dim3(2, U), kCompactThreads, 0, st, 0, true, kc, vc, nk, nv, c->len, B, N, c->kept_idx, c->first_evicted,
                        c->status));
+    if (c->wide_single) c->anchor_par ^= 1;
     c->anchor_valid = true;
     return KEYDIFF_OK;
 }

@@ -29,7 +29,7 @@ static_assert(kWideThreads == kSelThreads, "wide_select runs the selector's 256 
 // grid = U.  Also clears wide_move's counter and flags (2 * kMaxSegments per unit).
 __global__ void __launch_bounds__(kWideThreads)
 wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int raw_anchor,
-                   double* __restrict__ anchor_sum, double* __restrict__ deltas, int ndeltas, float* __restrict__ mu,
+                   const double* sum_in, double* sum_out /* may be the same */, double* __restrict__ deltas, int ndeltas, float* __restrict__ mu,
                    unsigned* __restrict__ move_sync) {
     __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     __shared__ float mu_sh[kHeadDim];
@@ -40,7 +40,7 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     if (u == 0 && tid == 2 * kMaxSegments) move_sync[0] = 0u;
     double run = 0.0;
     if (tid < kHeadDim) {
-        run = anchor_sum[static_cast<size_t>(u) * kHeadDim + tid];
+        run = sum_in[static_cast<size_t>(u) * kHeadDim + tid];
         // what the CTAs of the cluster kernel left beside the sum, in the order in which that kernel adds it
         if (deltas)
             for (int c = 0; c < ndeltas; ++c) {
@@ -52,7 +52,7 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     const double sum = run + block_sum_of_terms<kWideTermsDeep>(B, [&](int r) { return blk + static_cast<size_t>(r) * kRowVec; }, 1.0f / eps,
                                                                 raw_anchor != 0, table, tid);
     if (tid < kHeadDim) {
-        anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum;
+        sum_out[static_cast<size_t>(u) * kHeadDim + tid] = sum;
         mu_sh[tid] = static_cast<float>(sum / static_cast<double>(n));
         mu[static_cast<size_t>(u) * kMuStride + tid] = mu_sh[tid];
     }

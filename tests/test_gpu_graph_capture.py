@@ -39,3 +39,38 @@ def test_captured_steps_match_eager_steps(U, N, B, path, slots):
             del g
         kd.close()
     assert all(torch.equal(a, b) for a, b in zip(*out))
+
+
+@pytest.mark.parametrize("sizes", [(64, 1), (1, 64), (1, 1), (1, 64, 1, 1)])
+def test_replayed_steps_go_on_like_eager_ones(sizes):
+    # units of the cluster kernel whose single evicted rows take four launches: an even number of steps, captured once and replayed,
+    # carries the anchor's sum on from replay to replay, whichever kind the steps are
+    U, N = 185, 2048
+    wl = synth.Workload("t", 1, 1, U, 128, N, 64, "outlier", N + 4 * 64, 62)
+    k0, v0, stream = synth.prefilled_cache(wl, "cuda")
+    start, blocks = [stream.next_block(b) for b in (64, 1, 64)], [stream.next_block(b) for b in sizes]
+    out = []
+    for captured in (False, True):
+        k, v = k0.clone(), v0.clone()
+        kd = KeyDiff(1, 1, U, 128, N, 64)
+        kd.set_len(N)
+        for b in start:
+            kd.evict(k, v, *b)
+        torch.cuda.synchronize()
+        if captured:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g):
+                for b in blocks:
+                    kd.evict(k, v, *b)
+            for _ in range(3):
+                g.replay()
+        else:
+            for b in blocks * 3:
+                kd.evict(k, v, *b)
+        torch.cuda.synchronize()
+        assert int(kd.scratch()["status"].item()) == 0
+        out.append([k, v, kd.scratch()["kept_idx"].clone(), kd.scratch()["scores"][:, :N + sizes[-1]].clone()])
+        if captured:
+            del g
+        kd.close()
+    assert all(torch.equal(a, b) for a, b in zip(*out))
