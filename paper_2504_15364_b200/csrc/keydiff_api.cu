@@ -509,7 +509,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
         ++c->steps_since_full;
     }
     KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum_out,
-                   c->anchor_delta, c->cluster, c->mu, c->move_sync));
+                   c->anchor_delta, c->anchor_delta ? c->cluster : 0, c->mu, c->move_sync));
     // parts of at least 256 rows, enough of them for several rounds of three blocks per SM
     const long long rows = 1LL * U * n;
     const int want = static_cast<int>(rows / (12LL * c->sm_count));

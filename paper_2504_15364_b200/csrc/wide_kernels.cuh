@@ -38,16 +38,18 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     const uint4* blk = new_k + static_cast<size_t>(u) * B * kRowVec;
     if (tid < 2 * kMaxSegments) move_sync[1 + u * 2 * kMaxSegments + tid] = 0u;
     if (u == 0 && tid == 2 * kMaxSegments) move_sync[0] = 0u;
-    double run = 0.0;
+    // the sum, and what the CTAs of the cluster kernel left beside it, all requested at once
+    double run = 0.0, left[kMaxCluster];
+    double* delta = deltas + (static_cast<size_t>(u) * ndeltas) * kHeadDim + tid;
     if (tid < kHeadDim) {
         run = sum_in[static_cast<size_t>(u) * kHeadDim + tid];
-        // what the CTAs of the cluster kernel left beside the sum, in the order in which that kernel adds it
-        if (deltas)
-            for (int c = 0; c < ndeltas; ++c) {
-                double& delta = deltas[(static_cast<size_t>(u) * ndeltas + c) * kHeadDim + tid];
-                run += delta;
-                delta = 0.0;
-            }
+#pragma unroll
+        for (int c = 0; c < kMaxCluster; ++c) left[c] = c < ndeltas ? delta[c * kHeadDim] : 0.0;
+#pragma unroll
+        for (int c = 0; c < kMaxCluster; ++c) {
+            run += left[c];   // (in the order in which that kernel adds it)
+            if (left[c] != 0.0) delta[c * kHeadDim] = 0.0;
+        }
     }
     const double sum = run + block_sum_of_terms<kWideTermsDeep>(B, [&](int r) { return blk + static_cast<size_t>(r) * kRowVec; }, 1.0f / eps,
                                                                 raw_anchor != 0, table, tid);
