@@ -490,6 +490,12 @@ bool single_evicted(const keydiff_ctx* c, int B) {
     return c->wide_single && c->len + B == c->cfg.budget + 1 && c->incremental && c->anchor_valid && c->steps_since_full < 1024;
 }
 
+bool capturing(cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) { cudaGetLastError(); return false; }   // (the launch will say what is wrong)
+    return status != cudaStreamCaptureStatusNone;
+}
+
 int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int B, cudaStream_t st) {
     using namespace kd;
     const int N = c->cfg.budget, n = c->len + B, U = c->U;
@@ -498,7 +504,10 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     // other, as that kernel does: steps captured in a graph go on from replay to replay whichever kernels serve them.
     double* sum = c->anchor_sum[c->anchor_par];
     double* sum_out = c->wide_single ? c->anchor_sum[c->anchor_par ^ 1] : sum;
-    if (!(c->incremental && c->anchor_valid && c->steps_since_full < 1024)) {   // (never a step of single_evicted)
+    // A captured step of a context that always runs here rebuilds the sum each time it is replayed: a graph replayed on a cache that was refilled
+    // meanwhile (keydiff_reset and appends, keydiff_set_len) cannot see that the carried sum is another cache's, and such
+    // contexts could always be replayed like that with the staged kernels.  It costs 240 of 1140 us on 256 units of 16512 rows.
+    if (!(c->incremental && c->anchor_valid && c->steps_since_full < 1024) || (c->wide && capturing(st))) {   // (never a step of single_evicted)
         const int rows_per_split = (c->len + c->splits - 1) / c->splits;
         KD_CUDA(launch(anchor_partial_kernel, dim3(c->splits, U), kStagedThreads, 0, st, 0, true, kc, nk, c->len, 0, N, c->eps, rows_per_split,
                        c->nmax, c->partial, static_cast<float*>(nullptr), raw));

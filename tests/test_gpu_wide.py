@@ -115,3 +115,37 @@ def test_single_evicted_rows_between_whole_blocks(U, N, window, raw):
     torch.cuda.synchronize()
     assert int(status) == 0 and torch.equal(kept, kd.scratch()["kept_idx"].cpu())
     kd.close()
+
+
+def test_a_captured_step_replayed_after_the_cache_was_refilled(monkeypatch):
+    # a graph cannot know that appends or a restored cache made the carried sum stale: captured steps of these contexts carry none
+    monkeypatch.setenv("KEYDIFF_CLUSTER_SIZE", "1")
+    U, N, B = 2, 1400, 32
+    wl = synth.Workload("t", 1, 1, U, 128, N, B, "drift", 3 * N, 75)
+    k, v, stream = synth.prefilled_cache(wl, "cuda")
+    kd = KeyDiff(1, 1, U, 128, N, B)
+    assert kd.launch_info()["path"] == binding.KEYDIFF_PATH_STAGED
+    kd.set_len(N)
+    for _ in range(2):
+        kd.evict(k, v, *stream.next_block(B))
+    nk, nv = (x.clone() for x in stream.next_block(B))
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        kd.evict(k, v, nk, nv)
+    kd.reset()
+    while kd.len < N:   # another sequence
+        kd.evict(k, v, *stream.next_block(min(B, N - kd.len)))
+    for _ in range(3):
+        for t, new in zip((nk, nv), stream.next_block(B)):
+            t.copy_(new)
+        pre_k, pre_v = bits(k), bits(v)
+        g.replay()
+        torch.cuda.synchronize()
+        sc = kd.scratch()
+        assert int(sc["status"].item()) == 0
+        compare.check_step(pre_k, pre_v, N, bits(nk), bits(nv), N, bits(k), bits(v), sc["scores"].cpu().numpy(), sc["kept_idx"].cpu().numpy(),
+                           n_threads=8)
+    check(kd, k, v, *stream.next_block(B), N, N)   # and an eager step after them
+    del g
+    kd.close()
