@@ -225,14 +225,13 @@ class Run:
 
 
 def roofline_of(run, moved, step_ms, workload, compaction):
-    from paper_2504_15364_b200 import binding  # noqa: F401
     peak, peak_src = measured_peak()
     a_step = algorithmic_bytes(run.wl, moved, run.slots)
     kern_ms = float(step_ms.mean())
     achieved = a_step / (kern_ms * 1e-3) / 1e9
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
             "traffic": NCU_TRAFFIC_BYTES.get((workload, compaction)), "peak_source": peak_src,
-            "kernel": ("slot_evict_kernel" if run.slots else "fused_evict_kernel") if run.fused else "staged chain (4 kernels)",
+            "kernel": run.kd.kernel_name(),
             "algorithmic_bytes_per_launch": a_step, "moved_rows_per_unit": moved,
             "kernel_ms": kern_ms, "kernel_ms_median": float(np.median(step_ms)),
             "frac_of_nominal_8TBs": achieved / NOMINAL_HBM_GBS}

@@ -99,8 +99,9 @@ enum {
     KEYDIFF_PATH_AUTO = 0,    /* one fused launch, or four (reported as KEYDIFF_PATH_STAGED) where a unit
                                  does not fit it or four are faster; many long units that evict a single
                                  row take four in that step */
-    KEYDIFF_PATH_STAGED = 1,  /* four launches: anchor partials, scores, select, compaction */
-    KEYDIFF_PATH_FUSED = 2    /* one launch, one thread-block cluster per unit; create fails
+    KEYDIFF_PATH_STAGED = 1,  /* four launches: anchor partials, scores, select, compaction; nothing but the
+                                 caches is carried from step to step */
+    KEYDIFF_PATH_FUSED = 2    /* one launch, one thread block or one cluster of them per unit; create fails
                                  with KEYDIFF_ERR_UNSUPPORTED if a unit cannot fit */
 };
 
@@ -210,7 +211,14 @@ KEYDIFF_API int keydiff_destroy(keydiff_ctx* ctx);
  * sum is rebuilt from all n rows on the first evicting step, after any append-only step,
  * keydiff_set_len or keydiff_reset, and every 1024 evicting steps.  With on == 0 every step rebuilds it.
  * REQUIREMENT with on != 0: between two keydiff_evict calls nobody else may change rows [0, len) of
- * k_cache; after changing them call keydiff_set_len(ctx, len).  KEYDIFF_PATH_STAGED ignores the setting.
+ * k_cache; after changing them call keydiff_set_len(ctx, len).  It holds for every ctx that was not created with
+ * KEYDIFF_PATH_STAGED, also where keydiff_get_launch_info reports that path; KEYDIFF_PATH_STAGED ignores the setting.
+ * Non-finite keys reach the sum and leave it unspecified until the next rebuild.
+ * Stream capture: a captured step keeps the anchor of the ctx as it was when it was captured.  A graph of evicting steps
+ * may be launched again as the continuation of itself (with KEYDIFF_PATH_AUTO or _FUSED an even number of steps in it: the
+ * sum alternates between two buffers); after keydiff_reset, keydiff_set_len or appends only graphs of
+ * KEYDIFF_PATH_STAGED and of contexts that report it, which rebuild the sum in every captured step.  With slot reuse the positions of
+ * the new tokens are those of the capture.
  * Errors: INVALID_ARG (NULL ctx).
  */
 KEYDIFF_API int keydiff_set_incremental(keydiff_ctx* ctx, int32_t on);
@@ -274,11 +282,16 @@ KEYDIFF_API int keydiff_set_positions(keydiff_ctx* ctx, const int32_t* pos_devic
  */
 KEYDIFF_API int keydiff_get_moved_rows(const keydiff_ctx* ctx, const unsigned long long** counter);
 
-/* Launch facts of the chosen path, for benchmarks: path actually used (KEYDIFF_PATH_*),
- * kernels launched per evicting step, cluster size (1 for the staged path).  With slot reuse on the fused
- * path a step that has to rebuild the running anchor sum (keydiff_set_incremental) launches two more. */
+/* Launch facts of the chosen path, for benchmarks: path actually used (KEYDIFF_PATH_*), kernels launched per
+ * evicting step, cluster size (1 where no cluster is used).  Not counted: with path STAGED reported for KEYDIFF_PATH_AUTO,
+ * and with slot reuse in clusters, a step that has to rebuild the running anchor sum (keydiff_set_incremental)
+ * launches two more; and with KEYDIFF_PATH_AUTO a context of many long units in token order, whose steps are one launch,
+ * makes four in a step that evicts a single row. */
 KEYDIFF_API int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* launches_per_step,
                             int32_t* cluster_size);
+
+/* Name of the kernel, or of the group of four, that serves an evicting step; never NULL ("" for a NULL ctx). */
+KEYDIFF_API const char* keydiff_get_kernel_name(const keydiff_ctx* ctx);
 
 /*
  * keydiff_evict_static -- the eviction step for callers that cannot allocate device memory.

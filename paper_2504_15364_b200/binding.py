@@ -28,7 +28,7 @@ KEYDIFF_COMPACT_ORDERED, KEYDIFF_COMPACT_SLOT_REUSE = 0, 1
 # every symbol include/keydiff.h declares
 EXPORTS = ["keydiff_create", "keydiff_evict", "keydiff_evict_host", "keydiff_destroy", "keydiff_reset",
            "keydiff_get_len", "keydiff_set_len", "keydiff_get_scratch", "keydiff_get_moved_rows",
-           "keydiff_get_launch_info", "keydiff_evict_static", "keydiff_set_incremental", "keydiff_get_positions",
+           "keydiff_get_launch_info", "keydiff_get_kernel_name", "keydiff_evict_static", "keydiff_set_incremental", "keydiff_get_positions",
            "keydiff_set_positions", "keydiff_selftest_bounded_wait", "keydiff_debug_fail_alloc",
            "keydiff_strerror", "keydiff_last_cuda_error"]
 
@@ -79,10 +79,11 @@ def load_library() -> ctypes.CDLL:
     lib.keydiff_get_launch_info.argtypes = [vp, i32p, i32p, i32p]
     lib.keydiff_evict_static.argtypes = [vp, vp, vp, vp, i32, i32, i32, i32, i32, ctypes.c_float, vp]
     lib.keydiff_strerror.argtypes = [ctypes.c_int]
-    lib.keydiff_strerror.restype = ctypes.c_char_p
+    lib.keydiff_get_kernel_name.argtypes = [vp]
+    lib.keydiff_strerror.restype = lib.keydiff_get_kernel_name.restype = ctypes.c_char_p
     lib.keydiff_last_cuda_error.argtypes = []
     for name in EXPORTS:
-        if name != "keydiff_strerror":
+        if name not in ("keydiff_strerror", "keydiff_get_kernel_name"):
             getattr(lib, name).restype = ctypes.c_int
     from . import _pycall
     address = lambda f: ctypes.cast(f, vp).value
@@ -230,6 +231,10 @@ class KeyDiff:
         a, b, c = ctypes.c_int32(), ctypes.c_int32(), ctypes.c_int32()
         _check(self._lib.keydiff_get_launch_info(self._ctx, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)))
         return {"path": a.value, "launches_per_step": b.value, "cluster_size": c.value}
+
+    def kernel_name(self) -> str:
+        """``keydiff_get_kernel_name``: the kernel that serves an evicting step."""
+        return self._lib.keydiff_get_kernel_name(self._ctx).decode()
 
     def close(self):
         if self._ctx:

@@ -657,6 +657,7 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
             if (c->wide_single) ok = ok && alloc_wide(c);
         } else if (cfg->path == KEYDIFF_PATH_AUTO && !slot_reuse(c) && wide_select_smem(c->nmax) <= kWideSelectSmem) {
             c->wide = true;
+            c->cluster = 1;   // (a plan for clusters may have been made and found slower)
             const size_t sum_bytes = sizeof(double) * U * kd::kHeadDim;
             ok = kd_malloc(&c->anchor_sum[0], sum_bytes) == cudaSuccess &&
                  alloc_wide(c) && cudaMemset(c->anchor_sum[0], 0, sum_bytes) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
@@ -890,6 +891,14 @@ int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* laun
     if (launches_per_step) *launches_per_step = ctx->path == KEYDIFF_PATH_FUSED ? 1 : 4;
     if (cluster_size) *cluster_size = ctx->cluster;
     return KEYDIFF_OK;
+}
+
+const char* keydiff_get_kernel_name(const keydiff_ctx* ctx) {
+    if (!ctx) return "";
+    if (ctx->unit_blocks) return "unit_evict_kernel";
+    if (ctx->slot_stream) return "slot_evict_kernel";
+    if (ctx->path == KEYDIFF_PATH_FUSED) return "fused_evict_kernel";
+    return ctx->wide ? "wide kernels (4 launches)" : "staged kernels (4 launches)";
 }
 
 const char* keydiff_strerror(int code) {

@@ -149,3 +149,18 @@ def test_a_captured_step_replayed_after_the_cache_was_refilled(monkeypatch):
     check(kd, k, v, *stream.next_block(B), N, N)   # and an eager step after them
     del g
     kd.close()
+
+
+@pytest.mark.parametrize("U,N,B,slots,path,kernel", [
+    (16, 9000, 100, 0, 0, "wide kernels (4 launches)"),   # could run in clusters of ten and is faster without
+    (2, 20000, 64, 0, 0, "wide kernels (4 launches)"), (2, 700, 64, 0, 1, "staged kernels (4 launches)"), (2, 5000, 64, 0, 0, "fused_evict_kernel"),
+    (8, 200, 20, 0, 0, "unit_evict_kernel"), (224, 2048, 128, 1, 0, "unit_evict_kernel"), (2, 5000, 64, 1, 0, "slot_evict_kernel")])
+def test_launch_info_reports_what_runs(U, N, B, slots, path, kernel):
+    kd = KeyDiff(1, 1, U, 128, N, B, path=path, compaction=slots)
+    info = kd.launch_info()
+    assert kd.kernel_name() == kernel
+    if "4 launches" in kernel:
+        assert info == {"path": binding.KEYDIFF_PATH_STAGED, "launches_per_step": 4, "cluster_size": 1}
+    else:
+        assert info["path"] == binding.KEYDIFF_PATH_FUSED and info["launches_per_step"] == 1
+    kd.close()
