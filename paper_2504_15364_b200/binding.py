@@ -13,7 +13,6 @@ import torch
 
 _PKG = Path(__file__).resolve().parent
 LIB_PATH = _PKG / "libkeydiff.so"
-PYCALL_PATH = _PKG / "_pycall.so"
 
 KEYDIFF_OK = 0
 KEYDIFF_ERR_INVALID_ARG, KEYDIFF_ERR_UNSUPPORTED, KEYDIFF_ERR_ALLOC = -1, -2, -3
@@ -49,7 +48,21 @@ class KeyDiffError(RuntimeError):
 
 
 _lib = None
-_fast = None   # (C entry of KeyDiff.evict, addresses of keydiff_evict and keydiff_get_len), set with _lib
+_fast = None   # (entry of KeyDiff.evict, addresses of keydiff_evict and keydiff_get_len), set with _lib
+_EVICT_TYPE = ctypes.CFUNCTYPE(ctypes.c_int, *[ctypes.c_void_p] * 5, *[ctypes.c_int32] * 4, ctypes.c_void_p)
+_GET_LEN_TYPE = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.POINTER(ctypes.c_int32))
+
+
+def _evict_ctypes(evict, get_len, ctx, dtype, budget, heads, dim, row, stream, *tensors):
+    """What the C entry (csrc/pycall.c) does, where it was not built: the new length, a negative status, or None for tensors that do not fit."""
+    if any(t.dtype is not dtype or not t.is_cuda or not t.is_contiguous() for t in tensors):
+        return None
+    block = tensors[2].numel() // row
+    if [t.numel() for t in tensors] != [budget * row] * 2 + [block * row] * 2:
+        return None
+    rc, length = _EVICT_TYPE(evict)(ctx, *(t.data_ptr() for t in tensors), budget, block, heads, dim, stream), ctypes.c_int32()
+    rc = rc or _GET_LEN_TYPE(get_len)(ctx, ctypes.byref(length))
+    return rc or length.value
 
 
 def load_library() -> ctypes.CDLL:
@@ -57,7 +70,7 @@ def load_library() -> ctypes.CDLL:
     global _lib, _fast
     if _lib is not None:
         return _lib
-    if not LIB_PATH.exists() or not PYCALL_PATH.exists():
+    if not LIB_PATH.exists():
         raise KeyDiffError(KEYDIFF_ERR_STATE, f"{LIB_PATH} not built: run `python -m paper_2504_15364_b200.build`")
     lib = ctypes.CDLL(str(LIB_PATH))
     vp, i32 = ctypes.c_void_p, ctypes.c_int32
@@ -85,9 +98,12 @@ def load_library() -> ctypes.CDLL:
     for name in EXPORTS:
         if name not in ("keydiff_strerror", "keydiff_get_kernel_name"):
             getattr(lib, name).restype = ctypes.c_int
-    from . import _pycall
+    try:
+        from ._pycall import evict as entry
+    except ImportError:   # built without Python's headers, or for another interpreter
+        entry = _evict_ctypes
     address = lambda f: ctypes.cast(f, vp).value
-    _fast = (_pycall.evict, address(lib.keydiff_evict), address(lib.keydiff_get_len))
+    _fast = (entry, address(lib.keydiff_evict), address(lib.keydiff_get_len))
     _lib = lib
     return lib
 

@@ -1,5 +1,5 @@
 """Build step: compile the CUDA sources in ``csrc/`` into ``libkeydiff.so`` (sm_100a only) and the binding's C entry into
-``_pycall.so``."""
+``_pycall.<ABI>.so``."""
 from __future__ import annotations
 
 import os
@@ -24,16 +24,21 @@ def _stale(lib: Path) -> bool:
     return any(p.stat().st_mtime > t for p in deps)
 
 
-PYCALL = PKG / "_pycall.so"   # CPython entry of KeyDiff.evict (argument marshalling in C)
+# CPython entry of KeyDiff.evict (argument marshalling in C); its name carries the interpreter's ABI, so that another one does not load it
+PYCALL = PKG / ("_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))
 
 
-def build_pycall(force: bool = False) -> Path:
-    """Compile _pycall.so in-tree if missing or older than its source."""
-    src = CSRC / "pycall.c"
+def build_pycall(force: bool = False) -> Path | None:
+    """Compile the C entry in-tree if missing or older than its source.  None without Python's headers: the binding then makes the same call
+    through ctypes."""
+    src, include = CSRC / "pycall.c", Path(sysconfig.get_paths()["include"])
+    (PKG / "_pycall.so").unlink(missing_ok=True)   # (named without the ABI before: any interpreter would load it)
+    if not (include / "Python.h").exists():
+        print(f"{include}/Python.h not found: KeyDiff.evict goes through ctypes", file=sys.stderr)
+        return None
     if force or not PYCALL.exists() or src.stat().st_mtime > PYCALL.stat().st_mtime:
         tmp = PYCALL.with_suffix(f".{os.getpid()}.tmp")
-        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", f"-I{sysconfig.get_paths()['include']}",
-                        str(src), "-o", str(tmp)], check=True)
+        subprocess.run([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", f"-I{include}", str(src), "-o", str(tmp)], check=True)
         os.replace(tmp, PYCALL)
     return PYCALL
 
