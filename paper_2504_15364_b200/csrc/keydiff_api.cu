@@ -361,10 +361,10 @@ int launch_slot_stream(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, co
 // Many small units: one block per unit (unit_kernel.cuh).
 constexpr int kSmemPerSm = 228 * 1024;   // shared memory of an SM; a block takes 1 KB beside its own
 using UnitKernel = void (*)(kd::UnitParams);
-UnitKernel unit_instance(const keydiff_ctx* c) {   // unit_depth 0: rows straight from global memory
+UnitKernel unit_instance(const keydiff_ctx* c) {   // unit_depth 0, and the ordered layout: rows straight from global memory
     using namespace kd;
-    if (slot_reuse(c)) return c->unit_depth > 0 ? unit_evict_kernel<true, true> : unit_evict_kernel<true, false>;
-    return c->unit_depth > 0 ? unit_evict_kernel<false, true> : unit_evict_kernel<false, false>;
+    if (!slot_reuse(c)) return unit_evict_kernel<false, false>;
+    return c->unit_depth > 0 ? unit_evict_kernel<true, true> : unit_evict_kernel<true, false>;
 }
 // Where the block per unit is the faster kernel (us a step on a B200, unit kernel against cluster kernel):
 //   ordered layout   short units: 300 x 364 rows 26 / 46, 3000 x 364 225 / 310, 1000 x 564 137 / 137; while two blocks per SM serve
@@ -648,11 +648,12 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
         if (c->unit_blocks || c->slot_stream || (!slot_reuse(c) && plan_fused(c, prop.multiProcessorCount) && !wide_is_faster(c))) {
             c->path = KEYDIFF_PATH_FUSED;
             const size_t sum_bytes = sizeof(double) * U * kd::kHeadDim;
-            ok = kd_malloc(&c->anchor_sum[0], sum_bytes) == cudaSuccess && kd_malloc(&c->anchor_sum[1], sum_bytes) == cudaSuccess &&
-                 kd_malloc(&c->anchor_delta, sizeof(double) * U * c->cluster * kd::kHeadDim) == cudaSuccess &&
-                 cudaMemset(c->anchor_sum[0], 0, sum_bytes) == cudaSuccess && cudaMemset(c->anchor_sum[1], 0, sum_bytes) == cudaSuccess &&
-                 cudaMemset(c->anchor_delta, 0, sizeof(double) * U * c->cluster * kd::kHeadDim) == cudaSuccess &&
-                 cudaDeviceSynchronize() == cudaSuccess;
+            ok = kd_malloc(&c->anchor_sum[0], sum_bytes) == cudaSuccess && cudaMemset(c->anchor_sum[0], 0, sum_bytes) == cudaSuccess;
+            if (!c->unit_blocks)   // (the block of a unit keeps its sum in place)
+                ok = ok && kd_malloc(&c->anchor_sum[1], sum_bytes) == cudaSuccess &&
+                     kd_malloc(&c->anchor_delta, sum_bytes * c->cluster) == cudaSuccess &&
+                     cudaMemset(c->anchor_sum[1], 0, sum_bytes) == cudaSuccess && cudaMemset(c->anchor_delta, 0, sum_bytes * c->cluster) == cudaSuccess;
+            ok = ok && cudaDeviceSynchronize() == cudaSuccess;
             c->wide_single = wide_serves_single(c);
             if (c->wide_single) ok = ok && alloc_wide(c);
         } else if (cfg->path == KEYDIFF_PATH_AUTO && !slot_reuse(c) && wide_select_smem(c->nmax) <= kWideSelectSmem) {
