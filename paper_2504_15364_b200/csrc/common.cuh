@@ -23,9 +23,10 @@ constexpr int kErrInternal = -8;   // KEYDIFF_ERR_INTERNAL
 // Programmatic dependent launch: every kernel of a step is launched with the attribute (launch() in keydiff_api.cu), waits here for the
 // kernels in front of it in the stream before it touches global memory, and is brought onto the SMs while the one in
 // front ends.  Only the launch latency overlaps: 0.5 to 2 us of every call (16 calls on 8 units of 640 rows 210 -> 174 us,
-// together with the cheaper host path).  No kernel lets its successor in before its own work is done: blocks that move in earlier
-// and wait cost the kernels that fill the SMs' shared memory 0.7-1.3 % of a step, and the four launches of a step on
-// 256 units of 16512 rows 1138 instead of 902 us.
+// together with the cheaper host path).  No kernel lets its successor in before its rows are moved (the append before it writes slot
+// positions, the cluster kernels before their last barrier; a successor waits for all of it): blocks that move in earlier and wait
+// cost the kernels that fill the SMs' shared memory 0.7-1.3 % of a step, and the four launches of a step on 256 units of 16512
+// rows 1138 instead of 902 us.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -375,8 +375,8 @@ UnitKernel unit_instance(const keydiff_ctx* c) {   // unit_depth 0, and the orde
 //                    rows, 8 x 564 14 / 15, 8 x 1064 18 / 15.  Beyond 4500 rows only with many rounds
 //                    of units: 600 x 8224 268 / 263, 1000 x 8224 377 / 388, 4096 x 8224 1381 / 1460.
 // The ring (rows through shared memory by the copy engine) needs shared memory that short units' blocks put to better use: 800 x
-// 1764 142 with it, 131 without; with at most two blocks per SM, or long units, it is what keeps HBM busy: 224 x 2176 45 / 48,
-// 200 x 4160 57 / 64, 512 x 8224 197 / 232.
+// 1764 142 with it, 131 without; with at most two blocks per SM, or long units, it is what keeps HBM busy: 224 x 2176 44 / 45,
+// 200 x 4160 59 / 64, 1000 x 8224 376 / 437, 2000 x 8224 697 / 826.
 bool plan_unit(keydiff_ctx* c) {
     using namespace kd;
     if (c->tune_cluster > 0 || c->cfg.max_block > kSlotMaxBlock) return false;

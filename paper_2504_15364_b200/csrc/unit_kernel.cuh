@@ -6,7 +6,9 @@
 //
 // What bounds it: three blocks per SM (80 registers, by launch bounds; at 64 registers and four blocks most shapes lose 3-10 %)
 // work through a chain of about 14 us for a unit of 300 rows: 1344 x 316 rows 188 -> 97 us a step, with slot reuse 165 -> 81.
-// Long units: HBM, at 85-88 % of its copy rate with slot reuse (512 x 8224 rows: 197 us, 172 at the full rate).
+// Long units: HBM, with slot reuse (1000 x 8224 rows 376 us, 335 at the copy rate; 2000 x 8224 697, 670).
+// The ring's 64 KB leave room for two blocks per SM: on 224 x 2176 rows the 224 blocks are all there at once, and the step is
+// one chain (143 MB of traffic in 44 us, issue slots 43 % busy).
 #pragma once
 #include "low_select.cuh"
 #include "row_terms.cuh"

@@ -1,5 +1,6 @@
-// Ordered layout for units that no cluster can hold on chip (budgets beyond about 12000 tokens): four launches per step, as in
-// the staged path, but with the anchor's sum carried from step to step, so that the keys are read twice and not three times.
+// Ordered layout for units that no cluster can hold on chip (budgets beyond about 12000 tokens), for many of those that only
+// clusters of ten or more hold, and for steps of many long units that evict one row: four launches per step, as in the staged
+// path, but with the anchor's sum carried from step to step, so that the keys are read twice and not three times.
 //
 //   wide_anchor   running sum of the cached rows + the block rows' terms = this step's anchor (App. B.1, first expression)
 //   wide_score    norm, dot product and score of every key in one pass (second expression)
@@ -80,7 +81,7 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
     const int g = threadIdx.x >> 3, t = threadIdx.x & 7;
     const int r0 = blockIdx.x * rows_per_part, r1 = min(n, r0 + rows_per_part);
     const float* m4 = mu + static_cast<size_t>(u) * kMuStride;
-    float2 w[8];   // w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight: the chains of row_dot in pairs
+    float2 w[8];   // w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight: the chains of lane_dot16 in pairs
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const float4 x = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h)), y = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h + 4));
@@ -104,7 +105,7 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
         float ss[kWideDeep];
         double dot[kWideDeep];
 #pragma unroll
-        for (int k = 0; k < kWideDeep; ++k) {   // row_sumsq and row_dot up to the exchange between the lanes, in packed pairs
+        for (int k = 0; k < kWideDeep; ++k) {   // lane_sumsq and lane_dot16 in packed pairs
             float x[16];
             unpack_row(a[k], b[k], x);
             float2 q = make_float2(0.f, 0.f), c0 = q, c1 = q;
