@@ -194,11 +194,14 @@ FusedKernel fused_instance(int reg_rows, int* built, bool one_pass = false, bool
     return few_pre ? fused_instance_of<true, 1>(reg_rows, built) : fused_instance_of<true, 4>(reg_rows, built);
 }
 
-// Lets a kernel be launched with up to kSmemLimit bytes of dynamic shared memory.  The limit belongs to the kernel on the device, not to a
-// context: it is always the same, so that a context created later for smaller units does not lower it under an earlier one.
+// Lets a kernel be launched with as much shared memory as a block may have, its static part included.  The limit belongs to the
+// kernel on the device, not to a context: it is always the same, so that a context created later for smaller units does not lower it
+// under an earlier one.
 template <typename Kernel>
-bool allow_shared_memory(Kernel kern, int bytes = kd::kSmemLimit) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+bool allow_shared_memory(Kernel kern) {
+    cudaFuncAttributes attr;
+    return cuda_ok(cudaFuncGetAttributes(&attr, kern)) &&
+           cuda_ok(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kd::kSmemLimit - static_cast<int>(attr.sharedSizeBytes)));
 }
 
 // Co-resident clusters of `C` CTAs of the kernel `kern` with `smem` bytes each.
@@ -570,7 +573,7 @@ int launch_staged(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const u
 bool alloc_wide(keydiff_ctx* c) {
     return kd_malloc(&c->mu, sizeof(float) * c->U * kd::kMuStride) == cudaSuccess &&
            kd_malloc(&c->move_sync, sizeof(unsigned) * (1 + c->U * 2 * kd::kMaxSegments)) == cudaSuccess &&
-           allow_shared_memory(kd::wide_move_kernel, kMoveSmem);
+           allow_shared_memory(kd::wide_move_kernel);
 }
 
 int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
@@ -633,12 +636,12 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
              cudaMemset(c->moved_rows, 0, sizeof(unsigned long long)) == cudaSuccess;
     }
     if (ok) {
-        ok = allow_shared_memory(kd::select_kernel, kMaxSelectSmem) && allow_shared_memory(kd::wide_select_kernel, kWideSelectSmem);
+        ok = allow_shared_memory(kd::select_kernel) && allow_shared_memory(kd::wide_select_kernel);
     }
     if (ok && cfg->compaction == KEYDIFF_COMPACT_SLOT_REUSE) {
         ok = kd_malloc(&c->pos, sizeof(int32_t) * U * cfg->budget) == cudaSuccess &&
              cudaMemset(c->pos, 0, sizeof(int32_t) * U * cfg->budget) == cudaSuccess &&
-             allow_shared_memory(kd::slot_place_kernel, kMaxSelectSmem);   // (8 bytes per row of a block: checked above)
+             allow_shared_memory(kd::slot_place_kernel);
     }
     if (ok) ok = cudaDeviceSynchronize() == cudaSuccess;
     if (ok && cfg->path != KEYDIFF_PATH_STAGED) {
@@ -1001,8 +1004,7 @@ int static_scratch_for_current_device(unsigned char** out) {
         if (major != 10) return KEYDIFF_ERR_UNSUPPORTED;
         void* addr = nullptr;
         KD_CUDA(cudaGetSymbolAddress(&addr, g_static_scratch));
-        KD_CUDA(cudaFuncSetAttribute(kd::select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSelectSmem));
-        KD_CUDA(cudaFuncSetAttribute(kd::wide_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWideSelectSmem));
+        if (!allow_shared_memory(kd::select_kernel) || !allow_shared_memory(kd::wide_select_kernel)) return KEYDIFF_ERR_CUDA;
         g_static_scratch_addr[dev] = static_cast<unsigned char*>(addr);
     }
     *out = g_static_scratch_addr[dev];

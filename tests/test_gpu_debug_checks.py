@@ -48,3 +48,12 @@ def test_debug_build_runs_clean_and_matches_the_product_build():
     build.build_library()
     build.build_library(debug_checks=True)
     assert run("debug") == run("product")
+
+
+def test_the_phase_stamp_build_times_the_phases():
+    # its kernels have static shared memory beside the dynamic part
+    build.build_library(phase_stamps=True)
+    r = subprocess.run([sys.executable, "-m", "paper_2504_15364_b200.phase_times", "--workload", "single_step_n512", "--steps", "3"],
+                       capture_output=True, text=True, timeout=600, cwd=ROOT, env={**os.environ, "PYTHONPATH": ROOT})
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert float(r.stdout.split("total")[1].split()[0]) > 0
