@@ -46,3 +46,8 @@ def check_steps(U, N, B, length, slots, steps=3, model="outlier", kernel=None, b
 @pytest.mark.parametrize("B", [1, 2, 15, 16, 17, 32, 33, 48, 49, 64, 65, 100])
 def test_rows_around_the_depths_of_the_terms(B, slots):
     check_steps(5, 130, B, 130, slots, kernel="unit_evict_kernel")
+
+
+@pytest.mark.parametrize("N,length", [(640, 640), (641, 641), (640, 636), (640, 637), (643, 640), (4, 4), (8, 1)])
+def test_slot_lists_written_four_entries_at_a_time_or_not(N, length):
+    check_steps(3, N, 4, length, True)
