@@ -10,9 +10,9 @@
 // The running sum cannot drift: a row's terms are the fixed bit pattern that the other kernels add and take out as well
 // (row_terms.cuh), added and subtracted in double.
 //
-// What bounds it: HBM.  256 units of 16512 keys, 5.4 GB of traffic a step: 902 us; before, in the staged kernels, 1280 us (anchor and
-// score pass 308 + 229, selection 66, compaction 684).  Now the score pass takes 172 us (6.3 TB/s), the selection 30, the
-// compaction 683 (6.3 TB/s).
+// What bounds it: HBM.  256 units of 16512 keys, 5.4 GB of traffic a step: 891 us; in the staged kernels 1280 us (anchor and
+// score pass 308 + 229, selection 66, compaction 684).  The score pass takes 172 us (6.3 TB/s), the selection 25, the
+// compaction 679 (6.3 TB/s, and the last units' keys from L2).
 #pragma once
 #include "low_select.cuh"
 #include "row_terms.cuh"
@@ -70,6 +70,26 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     }
 }
 
+// lane_sumsq and lane_dot16 in packed pairs.  w: w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight, i.e. the
+// chains of lane_dot16.
+__device__ __forceinline__ void anchor_pairs(const float4& x, const float4& y, float2* w) {
+    w[0] = make_float2(x.x, y.x); w[1] = make_float2(x.y, y.y); w[2] = make_float2(x.z, y.z); w[3] = make_float2(x.w, y.w);
+}
+__device__ __forceinline__ void lane_sumsq_dot_pairs(const uint4& a, const uint4& b, const float2 (&w)[8], float& ss, double& dot) {
+    float x[16];
+    unpack_row(a, b, x);
+    float2 q = make_float2(0.f, 0.f), c0 = q, c1 = q;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) { const float2 v = make_float2(x[j], x[8 + j]); q = __ffma2_rn(v, v, q); }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        c0 = __ffma2_rn(make_float2(x[j], x[4 + j]), w[j], c0);
+        c1 = __ffma2_rn(make_float2(x[8 + j], x[12 + j]), w[4 + j], c1);
+    }
+    ss = q.x + q.y;
+    dot = (static_cast<double>(c0.x) + static_cast<double>(c0.y)) + (static_cast<double>(c1.x) + static_cast<double>(c1.y));
+}
+
 // One pass over the keys.  grid = (parts, U), rows_per_part a multiple of 128.  Four rows of a row group are requested
 // together: 32 KB in flight per block, three blocks per SM, which HBM's latency needs (with one row at a time, 8 KB per
 // block, and every lane finishing its row by itself the pass over 1.08 GB took 229 us; now 172).
@@ -81,13 +101,10 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
     const int g = threadIdx.x >> 3, t = threadIdx.x & 7;
     const int r0 = blockIdx.x * rows_per_part, r1 = min(n, r0 + rows_per_part);
     const float* m4 = mu + static_cast<size_t>(u) * kMuStride;
-    float2 w[8];   // w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight: the chains of lane_dot16 in pairs
+    float2 w[8];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const float4 x = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h)), y = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h + 4));
-        w[4 * h] = make_float2(x.x, y.x); w[4 * h + 1] = make_float2(x.y, y.y);
-        w[4 * h + 2] = make_float2(x.z, y.z); w[4 * h + 3] = make_float2(x.w, y.w);
-    }
+    for (int h = 0; h < 2; ++h)
+        anchor_pairs(*reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h)), *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h + 4)), w + 4 * h);
     const float m = m4[kHeadDim];
     float* out = scores + static_cast<size_t>(u) * nmax;
 #pragma unroll 1
@@ -105,20 +122,7 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
         float ss[kWideDeep];
         double dot[kWideDeep];
 #pragma unroll
-        for (int k = 0; k < kWideDeep; ++k) {   // lane_sumsq and lane_dot16 in packed pairs
-            float x[16];
-            unpack_row(a[k], b[k], x);
-            float2 q = make_float2(0.f, 0.f), c0 = q, c1 = q;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) { const float2 v = make_float2(x[j], x[8 + j]); q = __ffma2_rn(v, v, q); }
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                c0 = __ffma2_rn(make_float2(x[j], x[4 + j]), w[j], c0);
-                c1 = __ffma2_rn(make_float2(x[8 + j], x[12 + j]), w[4 + j], c1);
-            }
-            ss[k] = q.x + q.y;
-            dot[k] = (static_cast<double>(c0.x) + static_cast<double>(c0.y)) + (static_cast<double>(c1.x) + static_cast<double>(c1.y));
-        }
+        for (int k = 0; k < kWideDeep; ++k) lane_sumsq_dot_pairs(a[k], b[k], w, ss[k], dot[k]);
         const float r = sqrtf(group_sum_of4(ss, t));
         const float e = eviction_score(static_cast<float>(group_sum_of4(dot, t)), m, r, eps);
         const int i = base + (2 * (t & 1) + ((t >> 1) & 1)) * kWideGroups + g;
@@ -126,8 +130,71 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
     }
 }
 
-// Exact top-N (ties keep the older token), the ascending kept-index list, and the evicted rows' terms off the running sum (if
-// one is kept).
+// The keys of a unit's scores into shared memory, by 256 threads; tokens from `scored` on get the largest possible key (sliding window, Sec. 3.2).
+// Four at a time where the rows of the scratch begin on 16 bytes: with the list below made by the same threads 256 x 16512 rows 900 -> 895 us a
+// step, 200 x 12064 533 -> 528.
+// The scores may have been written in the same launch, by other SMs: they are read past L1.
+__device__ __forceinline__ void load_keys(const float* sc, int n, int scored, bool quads, uint32_t* keys, int tid) {
+    if (quads) {   // the row begins on 16 bytes, and so does the next: the last quad's end is padding
+        const float4* sc4 = reinterpret_cast<const float4*>(sc);
+        uint4* k4 = reinterpret_cast<uint4*>(keys);
+#pragma unroll 4
+        for (int q = tid; 4 * q < n; q += kSelThreads) {
+            const float4 e = __ldcg(&sc4[q]);
+            const int i = 4 * q;
+            k4[q] = make_uint4(i < scored ? order_key(e.x) : 0xffffffffu, i + 1 < scored ? order_key(e.y) : 0xffffffffu,
+                               i + 2 < scored ? order_key(e.z) : 0xffffffffu, i + 3 < scored ? order_key(e.w) : 0xffffffffu);
+        }
+    } else {
+#pragma unroll 8
+        for (int i = tid; i < n; i += kSelThreads) keys[i] = i < scored ? order_key(__ldcg(&sc[i])) : 0xffffffffu;
+    }
+}
+// Behind the selection, by 256 threads: tokens evicted in front of every word of the bitmap (n of them in all), and their list, ascending;
+// list may lie where the keys were.  Returns the first evicted token (E >= 1).
+__device__ __forceinline__ int list_evicted(int n, int tid, const Selector& s, int* before, int* list) {
+    const int nwords = (n + 31) >> 5;
+    const int per = (nwords + kSelThreads - 1) / kSelThreads, w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
+    int cnt = 0;
+    for (int q = w0; q < w1; ++q) cnt += __popc(s.bitmap[q]);
+    int run = sel_exclusive_scan(cnt, tid, s.wtot);
+    for (int q = w0; q < w1; ++q) {
+        before[q] = run;
+        for (uint32_t wd = s.bitmap[q]; wd; wd &= wd - 1) list[run++] = 32 * q + __ffs(wd) - 1;
+    }
+    __syncthreads();
+    return list[0];
+}
+// The kept-index list (ascending) and the evicted rows' terms off the running sum, if one is kept.  table: [8][128] doubles.
+__device__ __forceinline__ void finish_unit(int u, int tid, const uint4* k_cache, const uint4* new_k, int len, int B, int N, float eps, int raw_anchor,
+                                            double* anchor_sum, int32_t* kept_idx, int32_t* mirror, int32_t* first_evicted,
+                                            unsigned long long* moved_rows, const Selector& s, int* before, int* gone, double* table) {
+    const int n = len + B, first = list_evicted(n, tid, s, before, gone);
+    double sum = 0.0;   // (requested in front of the rows)
+    if (anchor_sum && tid < kHeadDim) sum = __ldcg(&anchor_sum[static_cast<size_t>(u) * kHeadDim + tid]);
+    if (tid == 0) {
+        first_evicted[u] = first;
+        // block rows always move into the cache, cache rows only from the first evicted one on
+        atomicAdd(moved_rows, static_cast<unsigned long long>(N - min(len, first)));
+    }
+    int32_t* out = kept_idx + static_cast<size_t>(u) * N;
+    int32_t* out2 = mirror ? mirror + static_cast<size_t>(u) * N : nullptr;
+#pragma unroll 4
+    for (int i = tid; i < n; i += kSelThreads) {
+        const uint32_t wd = s.bitmap[i >> 5], bit = 1u << (i & 31);
+        if (!(wd & bit)) {
+            const int d = i - before[i >> 5] - __popc(wd & (bit - 1u));
+            out[d] = i;
+            if (out2) out2[d] = i;
+        }
+    }
+    if (!anchor_sum) return;   // (the staged path keeps no sum)
+    const double terms = block_sum_of_terms<kWideTermsDeep>(n - N, [&](int r) { return concat_row(k_cache, new_k, u, gone[r], len, B, N); },
+                                                            1.0f / eps, raw_anchor != 0, table, tid);
+    if (tid < kHeadDim) anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum - terms;
+}
+
+// Exact top-N of a unit (ties keep the older token), its kept-index list, and the evicted rows' terms off the running sum.
 // grid = U; dynamic shared memory: n keys (padded to four), two bitmaps.
 __global__ void __launch_bounds__(kSelThreads)
 wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ new_k, const float* __restrict__ scores,
@@ -137,47 +204,15 @@ wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ 
     __shared__ __align__(128) SelectorScratch scratch;
     __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     grid_dependency_wait();
-    const int u = blockIdx.x, tid = threadIdx.x, n = len + B, E = n - N, nwords = (n + 31) >> 5;
+    const int u = blockIdx.x, tid = threadIdx.x, n = len + B, nwords = (n + 31) >> 5;
     uint32_t* keys = reinterpret_cast<uint32_t*>(smem);
     uint32_t* bitmap = keys + ((n + 3) & ~3);
     Selector s(scratch, bitmap, bitmap + nwords);
-    // sliding window (Sec. 3.2): the last `window` tokens carry the largest possible key
-    const float* sc = scores + static_cast<size_t>(u) * nmax;
-#pragma unroll 8
-    for (int i = tid; i < n; i += kSelThreads) keys[i] = i >= n - window ? 0xffffffffu : order_key(sc[i]);
+    load_keys(scores + static_cast<size_t>(u) * nmax, n, n - window, (nmax & 3) == 0, keys, tid);
     __syncthreads();
-    select_evicted(keys, n, E, tid, s);
-    // tokens evicted in front of every word
-    int* before = reinterpret_cast<int*>(s.eq);
-    const int per = (nwords + kSelThreads - 1) / kSelThreads, w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
-    int cnt = 0;
-    if (tid == 0) s.misc[1] = n;
-    for (int q = w0; q < w1; ++q) cnt += __popc(bitmap[q]);
-    int run = sel_exclusive_scan(cnt, tid, s.wtot);
-    uint32_t* gone = keys;   // the evicted tokens, ascending (the keys are dead)
-    for (int q = w0; q < w1; ++q) {
-        before[q] = run;
-        for (uint32_t wd = bitmap[q]; wd; wd &= wd - 1) {
-            const int i = 32 * q + __ffs(wd) - 1;
-            if (run == 0) s.misc[1] = i;
-            gone[run++] = static_cast<uint32_t>(i);
-        }
-    }
-    __syncthreads();
-    if (tid == 0) {
-        first_evicted[u] = s.misc[1];
-        // block rows always move into the cache, cache rows only from the first evicted one on
-        atomicAdd(moved_rows, static_cast<unsigned long long>(N - min(len, s.misc[1])));
-    }
-    int32_t* out = kept_idx + static_cast<size_t>(u) * N;
-    for (int i = tid; i < n; i += kSelThreads) {
-        const uint32_t wd = bitmap[i >> 5], bit = 1u << (i & 31);
-        if (!(wd & bit)) out[i - before[i >> 5] - __popc(wd & (bit - 1u))] = i;
-    }
-    if (!anchor_sum) return;   // (the staged path keeps no sum)
-    const double sum = block_sum_of_terms<kWideTermsDeep>(E, [&](int r) { return concat_row(k_cache, new_k, u, static_cast<int>(gone[r]), len, B, N); },
-                                                          1.0f / eps, raw_anchor != 0, table, tid);
-    if (tid < kHeadDim) anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] -= sum;
+    select_evicted(keys, n, n - N, tid, s);
+    finish_unit(u, tid, k_cache, new_k, len, B, N, eps, raw_anchor, anchor_sum, kept_idx, nullptr, first_evicted, moved_rows, s,
+                reinterpret_cast<int*>(s.eq), reinterpret_cast<int*>(keys), table);
 }
 
 // Step a4 in place by `segments` blocks per (unit, tensor): compact_kernel gives a tensor of a unit one block, which for fewer

@@ -51,3 +51,9 @@ def test_rows_around_the_depths_of_the_terms(B, slots):
 @pytest.mark.parametrize("N,length", [(640, 640), (641, 641), (640, 636), (640, 637), (643, 640), (4, 4), (8, 1)])
 def test_slot_lists_written_four_entries_at_a_time_or_not(N, length):
     check_steps(3, N, 4, length, True)
+
+
+@pytest.mark.parametrize("N,B,window", [(1301, 131, 0), (1300, 131, 40), (1298, 2, 7), (1300, 4, 1300 - 3)])
+def test_scores_read_four_at_a_time_or_not(monkeypatch, N, B, window):
+    monkeypatch.setenv("KEYDIFF_CLUSTER_SIZE", "1")   # units of this size then take the launches for long units
+    check_steps(2, N, B, N, False, blocks=[B, B, max(B - 1, 1)], kernel="wide kernels (4 launches)", recent_window=window)
