@@ -90,7 +90,8 @@ enum {
     KEYDIFF_COMPACT_SLOT_REUSE = 1  /* kept cache rows stay in their slots; the kept block rows take the
                                        freed slots: at most block_B rows per tensor are written.  The fused
                                        path serves it with one block per unit or with a streaming kernel in
-                                       clusters for max_block <= 1024; larger blocks go to the staged kernels (KEYDIFF_PATH_FUSED then fails with
+                                       clusters for max_block <= 1024, with KEYDIFF_PATH_AUTO also with several blocks per
+                                       unit (two launches); larger blocks go to the staged kernels (KEYDIFF_PATH_FUSED then fails with
                                        KEYDIFF_ERR_UNSUPPORTED) */
 };
 
@@ -284,8 +285,8 @@ KEYDIFF_API int keydiff_get_moved_rows(const keydiff_ctx* ctx, const unsigned lo
 
 /* Launch facts of the chosen path, for benchmarks: path actually used (KEYDIFF_PATH_*), kernels launched per
  * evicting step, cluster size (1 where no cluster is used).  Not counted: with path STAGED reported for KEYDIFF_PATH_AUTO,
- * and with slot reuse in clusters, a step that has to rebuild the running anchor sum (keydiff_set_incremental)
- * launches two more; and with KEYDIFF_PATH_AUTO a context of many long units in token order, whose steps are one launch,
+ * and with slot reuse in clusters or with several blocks per unit, a step that has to rebuild the running anchor sum (keydiff_set_incremental)
+ * launches up to two more; and with KEYDIFF_PATH_AUTO a context of many long units in token order, whose steps are one launch,
  * makes four in a step that evicts a single row. */
 KEYDIFF_API int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* launches_per_step,
                             int32_t* cluster_size);

@@ -16,6 +16,7 @@
 #include "slot_kernel.cuh"
 #include "unit_kernel.cuh"
 #include "wide_kernels.cuh"
+#include "parts_kernel.cuh"
 
 namespace {
 
@@ -83,6 +84,8 @@ struct keydiff_ctx {
     double* anchor_delta = nullptr;               // [U][cluster][128]
     bool wide = false;                            // ordered layout, no cluster holds a unit: wide_kernels.cuh on anchor_sum[0]
     bool wide_single = false;                     // ordered layout, cluster kernel: steps that evict one row go to wide_kernels.cuh
+    bool parts = false;                           // slot reuse: several blocks per unit serve a step (parts_kernel.cuh, on anchor_sum[0])
+    unsigned* parts_done = nullptr;               // [U] zero between steps
     float* mu = nullptr;                          // [U][kMuStride], the running step's anchors
     unsigned* move_sync = nullptr;                // [1 + U * 2 * kMaxSegments] counter and flags of wide_move_kernel
     float eps = kDefaultEps;
@@ -123,7 +126,7 @@ void free_scratch(keydiff_ctx* c) {
     }
     if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
     cudaFree(c->anchor_sum[0]); cudaFree(c->anchor_sum[1]); cudaFree(c->anchor_delta); cudaFree(c->pos);
-    cudaFree(c->mu); cudaFree(c->move_sync);
+    cudaFree(c->mu); cudaFree(c->move_sync); cudaFree(c->parts_done);
 }
 
 int check_step_args(const keydiff_ctx* ctx, const void* k_cache, const void* v_cache,
@@ -521,7 +524,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
         ++c->steps_since_full;
     }
     KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum_out,
-                   c->anchor_delta, c->anchor_delta ? c->cluster : 0, c->mu, c->move_sync));
+                   c->anchor_delta, c->anchor_delta ? c->cluster : 0, c->mu, c->move_sync, false));
     // parts of at least 256 rows, enough of them for several rounds of three blocks per SM
     const long long rows = 1LL * U * n;
     const int want = static_cast<int>(rows / (12LL * c->sm_count));
@@ -541,6 +544,68 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
         KD_CUDA(launch(compact_kernel, dim3(2, U), kCompactThreads, 0, st, 0, true, kc, vc, nk, nv, c->len, B, N, c->kept_idx, c->first_evicted,
                        c->status));
     if (c->wide_single) c->anchor_par ^= 1;
+    c->anchor_valid = true;
+    return KEYDIFF_OK;
+}
+
+// Slot reuse: where several blocks per unit are the faster way.  A block per unit (or, in slot_evict_kernel, a unit and round) is at its best
+// when its last round of units is full; fill = the share of the places of all rounds that have a unit.  Us a step, the other kernel
+// against parts (64 rows a block):
+//   up to 4500 rows   more than three units per SM and fill up to 0.77: 512 x 2112 84 / 75, 1000 x 2112 135 / 131, 900 x 4160 212 / 187,
+//                     1000 x 4160 225 / 205; 700 x 2112 (fill 0.79) 96 / 97, 400 x 4160 (0.9) 87 / 96.  Hardly more units than SMs: 160 x 4160
+//                     58 / 49, 180 x 2112 37 / 35; 224 x 2112 38 / 42.  Under 2000 rows the chain decides: 1000 x 1164 92 / 94.
+//   up to 10000       everywhere (150 x 8256 109 / 73, 240 x 8256 109 / 103, 512 x 8256 222 / 196, 1500 x 8256 563 / 534) but with nearly two units per
+//                     SM (256 x 8320, 128 rows a block 115 / 118), and with very many units, where HBM bounds both.
+//   beyond            two blocks per SM instead of three: fill up to 0.7: 160 x 16448 182 / 145, 300 x 20064 357 / 325; 400 x 16448 302 / 326.
+//   up to an SM's worth of units a step is one chain, and this one is longer: 130 x 8256 59 / 67, 64 x 4160 26 / 28.
+bool parts_are_faster(const keydiff_ctx* c) {
+    const int U = c->U, sms = c->sm_count, n = c->nmax;
+    if (c->cfg.path != KEYDIFF_PATH_AUTO || !slot_reuse(c) || c->tune_cluster > 0 || c->cfg.max_block > kd::kSlotMaxBlock || U <= sms || n < 2000 ||
+        2 * (kd::parts_layout(n, c->cfg.max_block).total + 1024) > kSmemPerSm)
+        return false;
+    const int at_once = c->unit_blocks ? (c->unit_depth > 0 ? 2 : 3) * sms : sms, rounds = (U + at_once - 1) / at_once;
+    const double fill = static_cast<double>(U) / (static_cast<double>(rounds) * at_once);
+    if (n > 10000) return fill <= 0.70;
+    if (n > 4500) return 10 * U <= 16 * sms || (U > 2 * sms && U <= 10 * sms);
+    return fill <= 0.77 && (10 * U <= 12 * sms || U > 3 * sms);
+}
+
+bool sum_valid(const keydiff_ctx* c) { return c->incremental && c->anchor_valid && c->steps_since_full < 1024; }
+
+// A block per unit rebuilds the sum by itself where that is needed.
+bool parts_serve(const keydiff_ctx* c) { return c->parts && (sum_valid(c) || !c->unit_blocks); }
+
+int launch_parts(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int B, cudaStream_t st) {
+    using namespace kd;
+    const int N = c->cfg.budget, n = c->len + B, U = c->U;
+    const bool raw = c->cfg.anchor_mode == KEYDIFF_ANCHOR_RAW_MEAN;
+    double* sum = c->anchor_sum[0];
+    if (!sum_valid(c)) {
+        const int rows_per_split = (c->len + c->splits - 1) / c->splits;
+        KD_CUDA(launch(anchor_partial_kernel, dim3(c->splits, U), kStagedThreads, 0, st, 0, true, kc, nk, c->len, 0, N, c->eps, rows_per_split,
+                       c->nmax, c->partial, static_cast<float*>(nullptr), raw));
+        KD_CUDA(launch(anchor_fold_kernel, dim3(U), kHeadDim, 0, st, 0, true, c->partial, c->splits, sum, static_cast<double*>(nullptr), 0));
+        c->steps_since_full = 0;
+    } else {
+        ++c->steps_since_full;
+    }
+    KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum, static_cast<double*>(nullptr), 0, c->mu,
+                   static_cast<unsigned*>(nullptr), true));
+    PartsParams q;
+    UnitParams& p = q.unit;
+    p.k_cache = kc; p.v_cache = vc; p.new_k = nk; p.new_v = nv;
+    p.len = c->len; p.B = B; p.N = N; p.nmax = c->nmax; p.max_block = c->cfg.max_block; p.eps = c->eps;
+    p.depth = 0; p.rebuild = 0;
+    p.scores = c->scores; p.kept_idx = c->kept_idx; p.first_evicted = c->first_evicted;
+    p.moved_rows = c->moved_rows; p.status = c->status;
+    p.anchor_sum = sum; p.raw_anchor = raw; p.window = c->cfg.recent_window;
+    p.pos = c->pos; p.next_pos = static_cast<int>(c->next_pos);
+    p.kept_mirror = c->kept_mirror;
+    q.mu = c->mu; q.parts_done = c->parts_done;
+    // a dozen parts per SM or more: 896 x 4352 rows 220 us a step, 227 with 512 rows a part; with fewer smaller ones: 224 x 2176 47 us, 50 with 1024
+    q.rows_per_part = 1LL * U * n >= 1024LL * 12 * c->sm_count ? 1024 : 512;
+    q.parts = (n + q.rows_per_part - 1) / q.rows_per_part;
+    KD_CUDA(launch(parts_kernel, dim3(q.parts, U), kUnitThreads, parts_layout(n, c->cfg.max_block).total, st, 0, true, q));
     c->anchor_valid = true;
     return KEYDIFF_OK;
 }
@@ -647,12 +712,16 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
     if (ok && cfg->path != KEYDIFF_PATH_STAGED) {
         // slot reuse is served by the streaming kernel (or, where that cannot hold a unit's keys, by the staged path)
         c->unit_blocks = plan_unit(c);
-        c->slot_stream = slot_reuse(c) && !c->unit_blocks && plan_slot_stream(c, prop.multiProcessorCount);
-        if (c->unit_blocks || c->slot_stream || (!slot_reuse(c) && plan_fused(c, prop.multiProcessorCount) && !wide_is_faster(c))) {
+        c->parts = parts_are_faster(c);
+        c->slot_stream = slot_reuse(c) && !c->unit_blocks && !c->parts && plan_slot_stream(c, prop.multiProcessorCount);
+        if (c->unit_blocks || c->parts || c->slot_stream || (!slot_reuse(c) && plan_fused(c, prop.multiProcessorCount) && !wide_is_faster(c))) {
             c->path = KEYDIFF_PATH_FUSED;
             const size_t sum_bytes = sizeof(double) * U * kd::kHeadDim;
             ok = kd_malloc(&c->anchor_sum[0], sum_bytes) == cudaSuccess && cudaMemset(c->anchor_sum[0], 0, sum_bytes) == cudaSuccess;
-            if (!c->unit_blocks)   // (the block of a unit keeps its sum in place)
+            if (c->parts)
+                ok = ok && kd_malloc(&c->mu, sizeof(float) * U * kd::kMuStride) == cudaSuccess && kd_malloc(&c->parts_done, sizeof(unsigned) * U) == cudaSuccess &&
+                     cudaMemset(c->parts_done, 0, sizeof(unsigned) * U) == cudaSuccess && allow_shared_memory(kd::parts_kernel);
+            else if (!c->unit_blocks)   // (a unit's block, or its last part, keeps its sum in place)
                 ok = ok && kd_malloc(&c->anchor_sum[1], sum_bytes) == cudaSuccess &&
                      kd_malloc(&c->anchor_delta, sum_bytes * c->cluster) == cudaSuccess &&
                      cudaMemset(c->anchor_sum[1], 0, sum_bytes) == cudaSuccess && cudaMemset(c->anchor_delta, 0, sum_bytes * c->cluster) == cudaSuccess;
@@ -723,7 +792,7 @@ int keydiff_evict(keydiff_ctx* ctx, void* k_cache, void* v_cache, const void* ne
         return KEYDIFF_OK;
     }
     const bool single = single_evicted(ctx, block_B);
-    const int lrc = ctx->path == KEYDIFF_PATH_FUSED && !single ? launch_fused(ctx, kc, vc, nk, nv, block_B, st)
+    const int lrc = parts_serve(ctx) ? launch_parts(ctx, kc, vc, nk, nv, block_B, st) : ctx->path == KEYDIFF_PATH_FUSED && !single ? launch_fused(ctx, kc, vc, nk, nv, block_B, st)
                      : ctx->wide || single              ? launch_wide(ctx, kc, vc, nk, nv, block_B, st)
                                                         : launch_staged(ctx, kc, vc, nk, nv, block_B, st);
     if (lrc != KEYDIFF_OK) return lrc;
@@ -892,13 +961,14 @@ int keydiff_get_moved_rows(const keydiff_ctx* ctx, const unsigned long long** co
 int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* launches_per_step, int32_t* cluster_size) {
     if (!ctx) return KEYDIFF_ERR_INVALID_ARG;
     if (path) *path = ctx->path;
-    if (launches_per_step) *launches_per_step = ctx->path == KEYDIFF_PATH_FUSED ? 1 : 4;
+    if (launches_per_step) *launches_per_step = ctx->parts ? 2 : ctx->path == KEYDIFF_PATH_FUSED ? 1 : 4;
     if (cluster_size) *cluster_size = ctx->cluster;
     return KEYDIFF_OK;
 }
 
 const char* keydiff_get_kernel_name(const keydiff_ctx* ctx) {
     if (!ctx) return "";
+    if (ctx->parts) return "parts_kernel";
     if (ctx->unit_blocks) return "unit_evict_kernel";
     if (ctx->slot_stream) return "slot_evict_kernel";
     if (ctx->path == KEYDIFF_PATH_FUSED) return "fused_evict_kernel";

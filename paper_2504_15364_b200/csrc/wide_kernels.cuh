@@ -27,18 +27,19 @@ constexpr int kMuStride = kHeadDim + 4;  // a unit's anchor and its norm
 static_assert(kWideDeep == 4, "group_sum_of4");
 static_assert(kWideThreads == kSelThreads, "wide_select runs the selector's 256 threads");
 
-// grid = U.  Also clears wide_move's counter and flags (2 * kMaxSegments per unit).
+// grid = U.  Also clears wide_move's counter and flags (2 * kMaxSegments per unit), if that is to follow.
 __global__ void __launch_bounds__(kWideThreads)
 wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int raw_anchor,
                    const double* sum_in, double* sum_out /* may be the same */, double* __restrict__ deltas, int ndeltas, float* __restrict__ mu,
-                   unsigned* __restrict__ move_sync) {
+                   unsigned* __restrict__ move_sync /* or nullptr */, bool let_in) {
     __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     __shared__ float mu_sh[kHeadDim];
     grid_dependency_wait();
+    if (let_in) grid_dependency_trigger();   // parts_kernel, which requests keys before it waits for the anchors
     const int u = blockIdx.x, tid = threadIdx.x;
     const uint4* blk = new_k + static_cast<size_t>(u) * B * kRowVec;
-    if (tid < 2 * kMaxSegments) move_sync[1 + u * 2 * kMaxSegments + tid] = 0u;
-    if (u == 0 && tid == 2 * kMaxSegments) move_sync[0] = 0u;
+    if (move_sync && tid < 2 * kMaxSegments) move_sync[1 + u * 2 * kMaxSegments + tid] = 0u;
+    if (move_sync && u == 0 && tid == 2 * kMaxSegments) move_sync[0] = 0u;
     // the sum, and what the CTAs of the cluster kernel left beside it, all requested at once
     double run = 0.0, left[kMaxCluster];
     double* delta = deltas + (static_cast<size_t>(u) * ndeltas) * kHeadDim + tid;

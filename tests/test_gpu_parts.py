@@ -1,0 +1,70 @@
+"""Slot reuse with several blocks per unit (csrc/parts_kernel.cuh): more units than SMs whose last round would be far from full, against the
+oracle; ragged parts, both variants, transition steps, blocks of one row, either way to the first sum, host entry and capture."""
+import pytest
+import torch
+
+from paper_2504_15364_b200 import KeyDiff, binding, synth
+from test_gpu_row_edges import check_steps
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("U,N,length,blocks,window,raw,model", [
+    (150, 2000, 2000, (128, 128, 1), 0, 0, "outlier"),            # a block per unit forms the first sum; 2128 = 4 parts of 512 and 80 rows
+    (177, 2047, 2000, (130, 130, 7), 400, 0, "clusters"),         # the first step also fills empty slots; single keys, window beyond the block
+    (160, 2304, 2304, (1, 256, 1, 255), 20, 1, "drift"),
+    (450, 1999, 1999, (3, 3), 0, 0, "offset"),
+    (150, 4600, 4600, (33, 33, 1), 0, 0, "outlier"),              # the first sum comes from launches of its own
+    (149, 10200, 10200, (64, 64), 0, 0, "drift")])                # two blocks per SM
+def test_steps_match_the_oracle(U, N, length, blocks, window, raw, model):
+    check_steps(U, N, max(blocks), length, True, model=model, kernel="parts_kernel", blocks=blocks, recent_window=window, anchor_mode=raw)
+
+
+@pytest.mark.parametrize("U,N,B,kernel", [(148, 2048, 128, "slot_evict_kernel"), (178, 2048, 128, "unit_evict_kernel"), (150, 1900, 64, "unit_evict_kernel"),
+                                          (237, 8192, 128, "slot_evict_kernel"), (236, 8192, 128, "parts_kernel"), (297, 8192, 128, "parts_kernel"),
+                                          (110, 12000, 64, "slot_evict_kernel"), (400, 12000, 64, "slot_evict_kernel"), (445, 2048, 64, "parts_kernel")])
+def test_which_kernel_serves(U, N, B, kernel):
+    kd = KeyDiff(1, 1, U, 128, N, B, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
+    assert kd.kernel_name() == kernel
+    info = kd.launch_info()
+    assert info["path"] == binding.KEYDIFF_PATH_FUSED and info["launches_per_step"] == (2 if kernel == "parts_kernel" else 1)
+    kd.close()
+
+
+@pytest.mark.parametrize("N", [2000, 4600])
+def test_captured_steps_and_the_host_entry_give_the_same(N):
+    U, B = 150, 64
+    wl = synth.Workload("t", 1, 1, U, 128, N, B, "outlier", N + 8 * B, 92)
+    k0, v0, stream = synth.prefilled_cache(wl, "cuda")
+    blocks = [stream.next_block(B) for _ in range(5)]
+    out = []
+    for way in ("eager", "captured", "host"):
+        k, v = k0.clone(), v0.clone()
+        kd = KeyDiff(1, 1, U, 128, N, B, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
+        kd.set_len(N)
+        kept = kd.scratch()["kept_idx"]
+        if way == "host":
+            kept, status = torch.zeros(U, N, dtype=torch.int32).pin_memory(), torch.ones(1, dtype=torch.int32).pin_memory()
+            for nk, nv in blocks:
+                kd.evict_host(k, v, nk.cpu().pin_memory(), nv.cpu().pin_memory(), kept, status)
+                torch.cuda.synchronize()
+            assert int(status) == 0
+        else:
+            kd.evict(k, v, *blocks[0])
+            torch.cuda.synchronize()
+            g = torch.cuda.CUDAGraph()
+            if way == "captured":
+                with torch.cuda.graph(g):
+                    for b in blocks[1:]:
+                        kd.evict(k, v, *b)
+                g.replay()
+            else:
+                for b in blocks[1:]:
+                    kd.evict(k, v, *b)
+            torch.cuda.synchronize()
+            del g
+        assert int(kd.scratch()["status"].item()) == 0
+        out.append([k, v, kept.cpu().clone(), kd.positions()[0].clone()])
+        kd.close()
+    for other in out[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(out[0], other))

@@ -48,9 +48,9 @@ def test_rows_around_the_depths_of_the_terms(B, slots):
     check_steps(5, 130, B, 130, slots, kernel="unit_evict_kernel")
 
 
-@pytest.mark.parametrize("N,length", [(640, 640), (641, 641), (640, 636), (640, 637), (643, 640), (4, 4), (8, 1)])
+@pytest.mark.parametrize("N,length", [(640, 640), (641, 641), (640, 636), (640, 637), (643, 640), (12, 4), (9, 1)])
 def test_slot_lists_written_four_entries_at_a_time_or_not(N, length):
-    check_steps(3, N, 4, length, True)
+    check_steps(3, N, 9, length, True)   # (more rows than there are empty slots: every step evicts)
 
 
 @pytest.mark.parametrize("N,B,window", [(1301, 131, 0), (1300, 131, 40), (1298, 2, 7), (1300, 4, 1300 - 3)])
