@@ -49,6 +49,10 @@ cudaError_t kd_malloc(void** p, size_t bytes) {
     return cudaMalloc(p, bytes);
 }
 template <typename T> cudaError_t kd_malloc(T** p, size_t bytes) { return kd_malloc(reinterpret_cast<void**>(p), bytes); }
+#ifdef KEYDIFF_DEBUG_CHECKS
+// Test hook of the debug-checks build (keydiff_debug_fail_launch): the n-th kernel launch from now on is not made and returns an error.
+int g_fail_launch_countdown = 0;
+#endif
 constexpr int kMaxSelectSmem = 200 * 1024;   // score keys of one unit must fit one CTA
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -144,6 +148,8 @@ int check_step_args(const keydiff_ctx* ctx, const void* k_cache, const void* v_c
 
 inline int prop_sm_count(const keydiff_ctx* c) { return c->sm_count > 0 ? c->sm_count : 148; }
 inline bool slot_reuse(const keydiff_ctx* c) { return c->cfg.compaction == KEYDIFF_COMPACT_SLOT_REUSE; }
+// The next step may go on from the running sum.
+inline bool sum_valid(const keydiff_ctx* c) { return c->incremental && c->anchor_valid && c->steps_since_full < 1024; }
 
 // Every kernel of a step goes through here: launched with programmatic stream serialization (it waits for the kernels in
 // front of it by itself, see grid_dependency_wait), as clusters of `cluster` blocks when that is not 0.  early = false: an
@@ -151,6 +157,9 @@ inline bool slot_reuse(const keydiff_ctx* c) { return c->cfg.compaction == KEYDI
 // be left without room for all of them at once (896 units of 4352 rows in clusters of five: +6 % of the step).
 template <typename... P, typename... A>
 cudaError_t launch(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, int cluster, bool early, A... args) {
+#ifdef KEYDIFF_DEBUG_CHECKS
+    if (g_fail_launch_countdown > 0 && --g_fail_launch_countdown == 0) return cudaErrorLaunchOutOfResources;
+#endif
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = dim3(threads);
@@ -307,7 +316,7 @@ bool plan_slot_stream(keydiff_ctx* c, int sm_count) {
 int launch_slot_stream(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int B, cudaStream_t st) {
     using namespace kd;
     const int N = c->cfg.budget, n = c->len + B;
-    if (!(c->incremental && c->anchor_valid && c->steps_since_full < 1024)) {
+    if (!sum_valid(c)) {
         // the running sum of the cached rows, rebuilt from all of them: first evicting step, after appends,
         // set_len / reset, periodically against rounding drift, and every step when the caller asked for it
         const int rows_per_split = (c->len + c->splits - 1) / c->splits;
@@ -413,7 +422,7 @@ int launch_unit(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     p.scores = c->scores; p.kept_idx = c->kept_idx; p.first_evicted = c->first_evicted;
     p.moved_rows = c->moved_rows; p.status = c->status;
     p.anchor_sum = c->anchor_sum[0];
-    p.rebuild = !(c->incremental && c->anchor_valid && c->steps_since_full < 1024);
+    p.rebuild = !sum_valid(c);
     p.raw_anchor = c->cfg.anchor_mode == KEYDIFF_ANCHOR_RAW_MEAN;
     p.window = c->cfg.recent_window;
     p.pos = c->pos; p.next_pos = static_cast<int>(c->next_pos);
@@ -438,7 +447,7 @@ int launch_fused(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const ui
     p.moved_rows = c->moved_rows; p.status = c->status;
     // The one-pass kernel needs the running anchor of the cache as it stands; every 1024 steps the
     // anchor is recomputed from all rows anyway, which sheds whatever rounding drift has built up.
-    const bool one_pass = c->incremental && c->anchor_valid && c->steps_since_full < 1024;
+    const bool one_pass = sum_valid(c);
     p.anchor_in = c->anchor_sum[c->anchor_par];
     p.anchor_out = c->anchor_sum[c->anchor_par ^ 1];
     p.anchor_delta = c->anchor_delta;
@@ -493,7 +502,7 @@ bool wide_serves_single(const keydiff_ctx* c) {
 }
 
 bool single_evicted(const keydiff_ctx* c, int B) {
-    return c->wide_single && c->len + B == c->cfg.budget + 1 && c->incremental && c->anchor_valid && c->steps_since_full < 1024;
+    return c->wide_single && c->len + B == c->cfg.budget + 1 && sum_valid(c);
 }
 
 bool capturing(cudaStream_t st) {
@@ -513,7 +522,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     // A captured step of a context that always runs here rebuilds the sum each time it is replayed: a graph replayed on a cache that was refilled
     // meanwhile (keydiff_reset and appends, keydiff_set_len) cannot see that the carried sum is another cache's, and such
     // contexts could always be replayed like that with the staged kernels.  It costs 240 of 1140 us on 256 units of 16512 rows.
-    if (!(c->incremental && c->anchor_valid && c->steps_since_full < 1024) || (c->wide && capturing(st))) {   // (never a step of single_evicted)
+    if (!sum_valid(c) || (c->wide && capturing(st))) {   // (never a step of single_evicted)
         const int rows_per_split = (c->len + c->splits - 1) / c->splits;
         KD_CUDA(launch(anchor_partial_kernel, dim3(c->splits, U), kStagedThreads, 0, st, 0, true, kc, nk, c->len, 0, N, c->eps, rows_per_split,
                        c->nmax, c->partial, static_cast<float*>(nullptr), raw));
@@ -523,6 +532,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     } else {
         ++c->steps_since_full;
     }
+    c->anchor_valid = false;   // until all launches of the step are made: one that fails leaves the sum, or the deltas, of a step half done
     KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum_out,
                    c->anchor_delta, c->anchor_delta ? c->cluster : 0, c->mu, c->move_sync, false));
     // parts of at least 256 rows, enough of them for several rounds of three blocks per SM
@@ -570,8 +580,6 @@ bool parts_are_faster(const keydiff_ctx* c) {
     return fill <= 0.77 && (10 * U <= 12 * sms || U > 3 * sms);
 }
 
-bool sum_valid(const keydiff_ctx* c) { return c->incremental && c->anchor_valid && c->steps_since_full < 1024; }
-
 // A block per unit rebuilds the sum by itself where that is needed.
 bool parts_serve(const keydiff_ctx* c) { return c->parts && (sum_valid(c) || !c->unit_blocks); }
 
@@ -589,6 +597,7 @@ int launch_parts(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const ui
     } else {
         ++c->steps_since_full;
     }
+    c->anchor_valid = false;   // (as in launch_wide)
     KD_CUDA(launch(wide_anchor_kernel, dim3(U), kWideThreads, 0, st, 0, true, nk, B, n, c->eps, raw, sum, sum, static_cast<double*>(nullptr), 0, c->mu,
                    static_cast<unsigned*>(nullptr), true));
     PartsParams q;
@@ -1000,6 +1009,12 @@ int keydiff_selftest_bounded_wait(int32_t* status_device, int32_t polls, void* s
 }
 
 #ifdef KEYDIFF_DEBUG_CHECKS
+__attribute__((visibility("default"))) int keydiff_debug_fail_launch(int32_t nth) {
+    if (nth < 0) return KEYDIFF_ERR_INVALID_ARG;
+    g_fail_launch_countdown = nth;
+    return KEYDIFF_OK;
+}
+
 // Debug-checks build only: the running sum of the cached rows' anchor terms as the latest step left it, [U][128] doubles, to out_host.
 // KEYDIFF_ERR_STATE when the next step would rebuild it.  Synchronises the device.
 __attribute__((visibility("default"))) int keydiff_debug_anchor_sum(const keydiff_ctx* ctx, double* out_host) {
