@@ -558,30 +558,51 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     return KEYDIFF_OK;
 }
 
-// Slot reuse: where several blocks per unit are the faster way.  A block per unit (or, in slot_evict_kernel, a unit and round) is at its best
-// when its last round of units is full; fill = the share of the places of all rounds that have a unit.  Us a step, the other kernel
-// against parts (64 rows a block):
-//   up to 4500 rows   more than three units per SM and fill up to 0.77: 512 x 2112 84 / 75, 1000 x 2112 135 / 131, 900 x 4160 212 / 187,
-//                     1000 x 4160 225 / 205; 700 x 2112 (fill 0.79) 96 / 97, 400 x 4160 (0.9) 87 / 96.  Hardly more units than SMs: 160 x 4160
-//                     58 / 49, 180 x 2112 37 / 35; 224 x 2112 38 / 42.  Under 2000 rows the chain decides: 1000 x 1164 92 / 94.
-//   up to 10000       everywhere (150 x 8256 109 / 73, 240 x 8256 109 / 103, 512 x 8256 222 / 196, 1500 x 8256 563 / 534) but with nearly two units per
-//                     SM (256 x 8320, 128 rows a block 115 / 118), and with very many units, where HBM bounds both.
-//   beyond            two blocks per SM instead of three: fill up to 0.7: 160 x 16448 182 / 145, 300 x 20064 357 / 325; 400 x 16448 302 / 326.
+// Slot reuse: where several blocks per unit are the faster way for a step of B rows.  Us a step, the kernel that serves otherwise / parts; rows a step in
+// brackets.  The lines are drawn so that of some 4700 shapes none loses more than 3 %, with blocks from one row to the largest that the context
+// takes.
+//   up to 4500 rows   otherwise a block per unit, at its best when its last round of units is full (fill: the share of the places of all rounds, three
+//                     per SM, that have a unit): 512 x 2112 (64) 84 / 75, 1000 x 2112 (64) 144 / 138, 900 x 4160 (64) 212 / 187; 700 x 2112 (64),
+//                     fill 0.79, 96 / 97.  Hardly more units than SMs: 160 x 2112 (64) 39 / 34, 177 x 2028 (128) 42 / 42; 224 x 2112 (64) 38 / 42.
+//                     Large blocks make one chain longer, which shows on short units: 160 x 2812 (512) 68 / 66, 177 x 2412 (512) 64 / 66, 149 x 2964
+//                     (1024) 97 / 102; 683 x 2284 (384), fill 0.77, 147 / 149, 600 x 2304 (256), 0.68, 126 / 122; 640 x 3828 (128) 160 /
+//                     148.  Budgets under 1940: 160 x 2006 (256) up 5 %.
+//   about 10000 rows  as long as three blocks of parts leave an SM its L1 (launch_parts): everywhere (150 x 8256 (64) 109 / 73, 236 x 8256 (64) 108 / 102, 512 x
+//                     8256 (64) 223 / 196, 400 x 8704 (512) 231 / 227, 1025 x 9216 (1024) 736 / 653) but with nearly two units per SM
+//                     (250 x 8448 (256) 127 / 132; the clusters are at their best with middling blocks, 236 x 4850 (200) 86 / 89, 400 x 6300 (200)
+//                     151 / 155), up to ten per SM (1480 x 8256 (64) 561 / 533; many more, and HBM bounds both).
+//   beyond            two blocks of parts per SM: hardly more units than one, two or three per SM: 160 x 16448 (64) 181 / 143, 183 x 12128 (128) 139 / 135, 345
+//                     x 16640 (256) 332 / 321, 460 x 14256 (256) 392 / 369; 207 x 12128 (128) 143 / 149, 560 x 10428 (128) 299 / 320; from 17700 rows
+//                     on earlier: 310 x 18128 (128) 353 / 325, 183 x 18128 (128) 195 / 203, 345 x 18128 (128) 335 / 359.
+//   blocks of > 512   take the clusters longer (400 x 10412 (512) 261, 400 x 10540 (640) 322), so that the lines lie further out: 190 x 12640 (640) 240 /
+//                     189, and there with 16 rows a step 132 / 125; 400 x 9916 (16) 188 / 179, but 400 x 11016 (16) 206 / 223.
 //   up to an SM's worth of units a step is one chain, and this one is longer: 130 x 8256 59 / 67, 64 x 4160 26 / 28.
-bool parts_are_faster(const keydiff_ctx* c) {
-    const int U = c->U, sms = c->sm_count, n = c->nmax;
-    if (c->cfg.path != KEYDIFF_PATH_AUTO || !slot_reuse(c) || c->tune_cluster > 0 || c->cfg.max_block > kd::kSlotMaxBlock || U <= sms || n < 2000 ||
-        2 * (kd::parts_layout(n, c->cfg.max_block).total + 1024) > kSmemPerSm)
+constexpr int kSmemBesideL1 = 196 * 1024;   // shared memory of an SM that leaves its L1 60 KB (the next larger split: 28)
+bool parts_are_faster(const keydiff_ctx* c, int B) {
+    const int U = c->U, sms = c->sm_count, n = c->nmax, N = c->cfg.budget, max_block = c->cfg.max_block;
+    if (c->cfg.path != KEYDIFF_PATH_AUTO || !slot_reuse(c) || c->tune_cluster > 0 || max_block > kd::kSlotMaxBlock || U <= sms || n < 2000 || N < 1940 ||
+        2 * (kd::parts_layout(n, max_block).total + 1024) > kSmemPerSm)
         return false;
-    const int at_once = c->unit_blocks ? (c->unit_depth > 0 ? 2 : 3) * sms : sms, rounds = (U + at_once - 1) / at_once;
-    const double fill = static_cast<double>(U) / (static_cast<double>(rounds) * at_once);
-    if (n > 10000) return fill <= 0.70;
-    if (n > 4500) return 10 * U <= 16 * sms || (U > 2 * sms && U <= 10 * sms);
-    return fill <= 0.77 && (10 * U <= 12 * sms || U > 3 * sms);
+    const auto within = [&](int from, int to) { return 100 * U > from * sms && 100 * U <= to * sms; };   // hundredths of a unit per SM
+    if (n <= 4500) {
+        const bool longer = N >= (B <= 512 ? 2600 : 3100);
+        if (U <= 2 * sms) return (B <= 512 || longer) && within(100, B <= 160 || longer ? 120 : 110);
+        const int rounds = (U + 3 * sms - 1) / (3 * sms);
+        const double fill = static_cast<double>(U) / (static_cast<double>(rounds) * 3 * sms);
+        return rounds > 1 && fill <= (B <= 64 || rounds > 2 || longer ? 0.77 : 0.70);
+    }
+    const bool large = max_block > 512, mid = max_block > 128 && max_block < 256;
+    if (3 * (kd::parts_layout(large && !c->unit_blocks ? N + 64 : n, max_block).total + 1024) <= kSmemBesideL1)
+        return within(100, mid && n <= 8000 ? 150 : 160) || (within(200, 1000) && !(mid && within(260, 296)));
+    if (n > 17700) return within(100, large ? 130 : 122) || within(200, large ? 233 : 210);
+    return within(100, large ? 135 : 124) || within(200, 233) || within(300, 311);
 }
 
-// A block per unit rebuilds the sum by itself where that is needed.
-bool parts_serve(const keydiff_ctx* c) { return c->parts && (sum_valid(c) || !c->unit_blocks); }
+// Whether the facts reported are those of several blocks per unit: a step of max_block rows.
+bool parts_named(const keydiff_ctx* c) { return c->parts && (!c->unit_blocks || parts_are_faster(c, c->cfg.max_block)); }
+
+// A block per unit rebuilds the sum by itself where that is needed, and goes on from the same sum.
+bool parts_serve(const keydiff_ctx* c, int B) { return c->parts && (!c->unit_blocks || (sum_valid(c) && parts_are_faster(c, B))); }
 
 int launch_parts(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uint4* nv, int B, cudaStream_t st) {
     using namespace kd;
@@ -614,7 +635,11 @@ int launch_parts(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const ui
     // a dozen parts per SM or more: 896 x 4352 rows 220 us a step, 227 with 512 rows a part; with fewer smaller ones: 224 x 2176 47 us, 50 with 1024
     q.rows_per_part = 1LL * U * n >= 1024LL * 12 * c->sm_count ? 1024 : 512;
     q.parts = (n + q.rows_per_part - 1) / q.rows_per_part;
-    KD_CUDA(launch(parts_kernel, dim3(q.parts, U), kUnitThreads, parts_layout(n, c->cfg.max_block).total, st, 0, true, q));
+    // Three blocks per SM have 98 KB of loads in flight, which L1 holds on their way: beyond kSmemBesideL1 it is down to 28 KB, and two blocks are faster than
+    // three (400 x 10156 rows, 256 a step, 251 us against 262; 177 x 12128, 128 a step, 132 against 139).  They are given more than they use.
+    int smem = parts_layout(n, c->cfg.max_block).total;
+    if (3 * (smem + 1024) > kSmemBesideL1) smem = std::max(smem, kSmemPerSm / 3);
+    KD_CUDA(launch(parts_kernel, dim3(q.parts, U), kUnitThreads, smem, st, 0, true, q));
     c->anchor_valid = true;
     return KEYDIFF_OK;
 }
@@ -721,7 +746,7 @@ int create_impl(const keydiff_config* cfg, keydiff_ctx** out) {
     if (ok && cfg->path != KEYDIFF_PATH_STAGED) {
         // slot reuse is served by the streaming kernel (or, where that cannot hold a unit's keys, by the staged path)
         c->unit_blocks = plan_unit(c);
-        c->parts = parts_are_faster(c);
+        c->parts = parts_are_faster(c, c->unit_blocks ? 1 : cfg->max_block);   // (a block per unit takes the steps that it is faster at)
         c->slot_stream = slot_reuse(c) && !c->unit_blocks && !c->parts && plan_slot_stream(c, prop.multiProcessorCount);
         if (c->unit_blocks || c->parts || c->slot_stream || (!slot_reuse(c) && plan_fused(c, prop.multiProcessorCount) && !wide_is_faster(c))) {
             c->path = KEYDIFF_PATH_FUSED;
@@ -801,7 +826,7 @@ int keydiff_evict(keydiff_ctx* ctx, void* k_cache, void* v_cache, const void* ne
         return KEYDIFF_OK;
     }
     const bool single = single_evicted(ctx, block_B);
-    const int lrc = parts_serve(ctx) ? launch_parts(ctx, kc, vc, nk, nv, block_B, st) : ctx->path == KEYDIFF_PATH_FUSED && !single ? launch_fused(ctx, kc, vc, nk, nv, block_B, st)
+    const int lrc = parts_serve(ctx, block_B) ? launch_parts(ctx, kc, vc, nk, nv, block_B, st) : ctx->path == KEYDIFF_PATH_FUSED && !single ? launch_fused(ctx, kc, vc, nk, nv, block_B, st)
                      : ctx->wide || single              ? launch_wide(ctx, kc, vc, nk, nv, block_B, st)
                                                         : launch_staged(ctx, kc, vc, nk, nv, block_B, st);
     if (lrc != KEYDIFF_OK) return lrc;
@@ -970,14 +995,14 @@ int keydiff_get_moved_rows(const keydiff_ctx* ctx, const unsigned long long** co
 int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* launches_per_step, int32_t* cluster_size) {
     if (!ctx) return KEYDIFF_ERR_INVALID_ARG;
     if (path) *path = ctx->path;
-    if (launches_per_step) *launches_per_step = ctx->parts ? 2 : ctx->path == KEYDIFF_PATH_FUSED ? 1 : 4;
+    if (launches_per_step) *launches_per_step = parts_named(ctx) ? 2 : ctx->path == KEYDIFF_PATH_FUSED ? 1 : 4;
     if (cluster_size) *cluster_size = ctx->cluster;
     return KEYDIFF_OK;
 }
 
 const char* keydiff_get_kernel_name(const keydiff_ctx* ctx) {
     if (!ctx) return "";
-    if (ctx->parts) return "parts_kernel";
+    if (parts_named(ctx)) return "parts_kernel";
     if (ctx->unit_blocks) return "unit_evict_kernel";
     if (ctx->slot_stream) return "slot_evict_kernel";
     if (ctx->path == KEYDIFF_PATH_FUSED) return "fused_evict_kernel";

@@ -15,14 +15,31 @@ pytestmark = pytest.mark.gpu
     (160, 2304, 2304, (1, 256, 1, 255), 20, 1, "drift"),
     (450, 1999, 1999, (3, 3), 0, 0, "offset"),
     (150, 4600, 4600, (33, 33, 1), 0, 0, "outlier"),              # the first sum comes from launches of its own
-    (149, 10200, 10200, (64, 64), 0, 0, "drift")])                # two blocks per SM
+    (149, 10200, 10200, (64, 64), 0, 0, "drift"),                 # two blocks per SM, though three would fit
+    (149, 13000, 13000, (64, 64), 0, 0, "outlier"),               # two fit
+    (450, 1950, 1950, (1023, 1, 1023), 0, 0, "offset"),           # three lists of blocks this large take more than the keys
+    (150, 3900, 3900, (700, 5, 700), 900, 0, "outlier")])
 def test_steps_match_the_oracle(U, N, length, blocks, window, raw, model):
     check_steps(U, N, max(blocks), length, True, model=model, kernel="parts_kernel", blocks=blocks, recent_window=window, anchor_mode=raw)
 
 
+@pytest.mark.parametrize("U,N,blocks,window", [(160, 2500, (600, 1, 600, 64, 512, 513), 0), (640, 1950, (384, 16, 384, 1), 500)])
+def test_a_block_per_unit_takes_the_large_blocks_of_a_context(U, N, blocks, window):
+    check_steps(U, N, max(blocks), N, True, model="offset", kernel="unit_evict_kernel", blocks=blocks, recent_window=window)
+
+
 @pytest.mark.parametrize("U,N,B,kernel", [(148, 2048, 128, "slot_evict_kernel"), (178, 2048, 128, "unit_evict_kernel"), (150, 1900, 64, "unit_evict_kernel"),
                                           (237, 8192, 128, "slot_evict_kernel"), (236, 8192, 128, "parts_kernel"), (297, 8192, 128, "parts_kernel"),
-                                          (110, 12000, 64, "slot_evict_kernel"), (400, 12000, 64, "slot_evict_kernel"), (445, 2048, 64, "parts_kernel")])
+                                          (110, 12000, 64, "slot_evict_kernel"), (400, 12000, 64, "slot_evict_kernel"), (445, 2048, 64, "parts_kernel"),
+                                          # large blocks, and where parts leave an SM no L1 or only two blocks: 3 to 15 % slower with several per unit
+                                          (149, 2048, 1024, "unit_evict_kernel"), (177, 2300, 512, "unit_evict_kernel"), (683, 1900, 384, "unit_evict_kernel"),
+                                          (600, 2048, 256, "parts_kernel"), (1000, 8192, 1024, "parts_kernel"), (400, 8192, 512, "parts_kernel"),
+                                          (400, 9700, 64, "parts_kernel"), (400, 9900, 256, "slot_evict_kernel"), (236, 9900, 256, "slot_evict_kernel"),
+                                          (400, 9900, 640, "parts_kernel"), (1000, 9900, 256, "unit_evict_kernel"), (330, 10156, 128, "parts_kernel"),
+                                          (200, 12000, 64, "slot_evict_kernel"), (190, 12000, 640, "parts_kernel"), (190, 18000, 16, "slot_evict_kernel"),
+                                          (177, 20000, 16, "parts_kernel"), (330, 18000, 16, "slot_evict_kernel"),
+                                          (236, 4650, 200, "slot_evict_kernel"), (222, 4650, 200, "parts_kernel"), (400, 6100, 200, "slot_evict_kernel"),
+                                          (1025, 9500, 640, "unit_evict_kernel"), (177, 3100, 256, "parts_kernel"), (149, 1910, 128, "unit_evict_kernel")])
 def test_which_kernel_serves(U, N, B, kernel):
     kd = KeyDiff(1, 1, U, 128, N, B, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
     assert kd.kernel_name() == kernel
