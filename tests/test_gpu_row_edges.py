@@ -48,6 +48,12 @@ def test_rows_around_the_depths_of_the_terms(B, slots):
     check_steps(5, 130, B, 130, slots, kernel="unit_evict_kernel")
 
 
+@pytest.mark.parametrize("B", [16, 17, 32, 33, 64, 65, 80, 81, 128, 129, 144, 193, 257])
+def test_rows_around_the_depths_of_the_long_units_terms(monkeypatch, B):
+    monkeypatch.setenv("KEYDIFF_CLUSTER_SIZE", "1")   # units of this size then take the launches for long units: up to eight rows together
+    check_steps(2, 1500, B, 1500, False, kernel="wide kernels (4 launches)", model="drift")
+
+
 @pytest.mark.parametrize("N,length", [(640, 640), (641, 641), (640, 636), (640, 637), (643, 640), (12, 4), (9, 1)])
 def test_slot_lists_written_four_entries_at_a_time_or_not(N, length):
     check_steps(3, N, 9, length, True)   # (more rows than there are empty slots: every step evicts)
