@@ -15,7 +15,11 @@ constexpr int kLanesPerRow = 8;            // a row is handled by 8 consecutive 
 // store is skipped.  Without the macro the check is not compiled.
 constexpr int kErrInternal = -8;   // KEYDIFF_ERR_INTERNAL
 #ifdef KEYDIFF_DEBUG_CHECKS
-#define KD_ROW_OK(d, limit, status) ((static_cast<unsigned>(d) < static_cast<unsigned>(limit)) || (atomicExch((status), kd::kErrInternal), false))
+#define KD_ROW_OK(d, limit, status) ((static_cast<unsigned>(d) < static_cast<unsigned>(limit)) || kd::bad_row(status))
+__device__ __forceinline__ bool bad_row(int32_t* status) {   // status may be nullptr (keydiff_evict_static has none)
+    if (status) atomicExch(status, kErrInternal);
+    return false;
+}
 #else
 #define KD_ROW_OK(d, limit, status) true
 #endif

@@ -542,7 +542,7 @@ int launch_wide(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const uin
     KD_CUDA(launch(wide_score_kernel, dim3((n + rows_per_part - 1) / rows_per_part, U), kWideThreads, 0, st, 0, true, kc, nk, c->len, B, N,
                    c->eps, rows_per_part, c->nmax, c->mu, c->scores));
     KD_CUDA(launch(wide_select_kernel, dim3(U), kSelThreads, wide_select_smem(n), st, 0, true, kc, nk, c->scores, c->len, B, N, c->eps, raw,
-                   c->nmax, c->cfg.recent_window, sum_out, c->kept_idx, c->first_evicted, c->moved_rows));
+                   c->nmax, c->cfg.recent_window, sum_out, c->kept_idx, c->first_evicted, c->moved_rows, c->status));
     // as many blocks as run at once, three per SM, of at least 512 rows each (150 x 10600 rows: 408 us with 300 blocks, 474
     // with 600; 100 x 10600: 318 with 200, 287 with 400, 328 with 600); one per unit and tensor when the rows that a
     // block reads ahead do not fit its shared memory
@@ -655,7 +655,7 @@ int launch_staged(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, const u
                    c->partial, c->norms, c->scores));
     if (!slot_reuse(c) && wide_select_smem(n) <= kWideSelectSmem)
         KD_CUDA(launch(wide_select_kernel, dim3(U), kSelThreads, wide_select_smem(n), st, 0, true, kc, nk, c->scores, c->len, B, N, c->eps, 0,
-                       c->nmax, c->cfg.recent_window, static_cast<double*>(nullptr), c->kept_idx, c->first_evicted, c->moved_rows));
+                       c->nmax, c->cfg.recent_window, static_cast<double*>(nullptr), c->kept_idx, c->first_evicted, c->moved_rows, c->status));
     else
         KD_CUDA(launch(select_kernel, dim3(U), kSelectThreads, static_cast<size_t>(n) * 4, st, 0, true, c->scores, n, N, c->nmax, c->len, c->kept_idx,
                        c->first_evicted, c->moved_rows, c->cfg.recent_window, slot_reuse(c) ? c->pos : nullptr,
@@ -1187,7 +1187,7 @@ extern "C" int keydiff_evict_static(void* k_cache, void* v_cache, const void* ne
     KD_CUDA(launch(score_kernel, grid, kStagedThreads, 0, st, 0, true, kc, nk, len, block_B, N, e, rows_per_split, nn, partial, norms, scores));
     if (wide_select_smem(nn) <= kWideSelectSmem)
         KD_CUDA(launch(wide_select_kernel, dim3(U), kSelThreads, wide_select_smem(nn), st, 0, true, kc, nk, scores, len, block_B, N, e, 0, nn, 0,
-                       static_cast<double*>(nullptr), kept, first, moved));
+                       static_cast<double*>(nullptr), kept, first, moved, static_cast<int32_t*>(nullptr)));
     else
         KD_CUDA(launch(select_kernel, dim3(U), kSelectThreads, static_cast<size_t>(nn) * 4, st, 0, true, scores, nn, N, nn, len, kept, first, moved, 0,
                        nullptr, 0));

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kUnitThreads, 3) parts_kernel(const PartsParam
     }
     select_evicted(keys, n, E, tid, s);
     int* ev_of = reinterpret_cast<int*>(keys);
-    const int first = list_evicted(n, tid, s, before, ev_of);
+    const int first = list_evicted(n, tid, s, before, ev_of, p.max_block, p.status);
     const double sum = tid < kHeadDim ? p.anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] : 0.0;
     place_block_rows<kWideTermsDeep>(p, u, tid, n, E, bitmap, before, ev_of, first, sum, 1.0f / p.eps, p.raw_anchor != 0, sums);
 }

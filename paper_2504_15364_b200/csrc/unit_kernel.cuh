@@ -10,7 +10,7 @@
 // The ring's 64 KB leave room for two blocks per SM: on 224 x 2176 rows the 224 blocks are all there at once, and the step is
 // one chain (143 MB of traffic in 44 us, issue slots 43 % busy).
 #pragma once
-#include "low_select.cuh"
+#include "evicted_list.cuh"
 #include "row_terms.cuh"
 #include "slot_kernel.cuh"      // issue_rows
 #include "staged_kernels.cuh"   // concat_row
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitP
     uint32_t* bitmap = reinterpret_cast<uint32_t*>(smem + L.bitmap);
     int* ev_of = reinterpret_cast<int*>(smem + L.lists);   // evicted candidates, ascending
     const int u = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, t = tid & 7, sub = lane >> 3;
-    const int len = p.len, B = p.B, N = p.N, n = len + B, E = n - N, nwords = (n + 31) >> 5;
+    const int len = p.len, B = p.B, N = p.N, n = len + B, E = n - N;
     const float inv_eps = 1.0f / p.eps;
     const bool raw = p.raw_anchor != 0;
     const int tiles = (n + kTileRows - 1) / kTileRows, D = p.depth;
@@ -217,22 +217,8 @@ __global__ void __launch_bounds__(kUnitThreads, 3) unit_evict_kernel(const UnitP
     select_evicted(keys, n, E, tid, s);
     auto evicted = [&](int i) { return ((bitmap[i >> 5] >> (i & 31)) & 1u) != 0; };
     int* before = reinterpret_cast<int*>(s.eq);   // evicted candidates in front of every word
-    {
-        const int per = (nwords + kUnitThreads - 1) / kUnitThreads, w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
-        int cnt = 0;
-        for (int q = w0; q < w1; ++q) cnt += __popc(bitmap[q]);
-        int run = sel_exclusive_scan(cnt, tid, s.wtot);
-        for (int q = w0; q < w1; ++q) {
-            before[q] = run;
-            for (uint32_t wd = bitmap[q]; wd; wd &= wd - 1) {
-                if (!KD_ROW_OK(run, p.max_block, p.status)) break;
-                ev_of[run++] = 32 * q + __ffs(wd) - 1;
-            }
-        }
-    }
-    __syncthreads();
+    const int first_evicted = list_evicted(n, tid, s, before, ev_of, p.max_block, p.status);
     auto evicted_before = [&](int i) { return before[i >> 5] + __popc(bitmap[i >> 5] & ((1u << (i & 31)) - 1u)); };
-    const int first_evicted = ev_of[0];   // (E >= 1)
     int32_t* kept = p.kept_idx + static_cast<size_t>(u) * N;
     int32_t* mirror = p.kept_mirror ? p.kept_mirror + static_cast<size_t>(u) * N : nullptr;
     if constexpr (!kSlots) {

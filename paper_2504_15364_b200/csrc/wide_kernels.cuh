@@ -14,7 +14,7 @@
 // score pass 308 + 229, selection 66, compaction 684).  The score pass takes 172 us (6.3 TB/s), the selection 25, the
 // compaction 679 (6.3 TB/s, and the last units' keys from L2).
 #pragma once
-#include "low_select.cuh"
+#include "evicted_list.cuh"
 #include "row_terms.cuh"
 #include "staged_kernels.cuh"
 
@@ -71,26 +71,6 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     }
 }
 
-// lane_sumsq and lane_dot16 in packed pairs.  w: w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight, i.e. the
-// chains of lane_dot16.
-__device__ __forceinline__ void anchor_pairs(const float4& x, const float4& y, float2* w) {
-    w[0] = make_float2(x.x, y.x); w[1] = make_float2(x.y, y.y); w[2] = make_float2(x.z, y.z); w[3] = make_float2(x.w, y.w);
-}
-__device__ __forceinline__ void lane_sumsq_dot_pairs(const uint4& a, const uint4& b, const float2 (&w)[8], float& ss, double& dot) {
-    float x[16];
-    unpack_row(a, b, x);
-    float2 q = make_float2(0.f, 0.f), c0 = q, c1 = q;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) { const float2 v = make_float2(x[j], x[8 + j]); q = __ffma2_rn(v, v, q); }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        c0 = __ffma2_rn(make_float2(x[j], x[4 + j]), w[j], c0);
-        c1 = __ffma2_rn(make_float2(x[8 + j], x[12 + j]), w[4 + j], c1);
-    }
-    ss = q.x + q.y;
-    dot = (static_cast<double>(c0.x) + static_cast<double>(c0.y)) + (static_cast<double>(c1.x) + static_cast<double>(c1.y));
-}
-
 // One pass over the keys.  grid = (parts, U), rows_per_part a multiple of 128.  Four rows of a row group are requested
 // together: 32 KB in flight per block, three blocks per SM, which HBM's latency needs (with one row at a time, 8 KB per
 // block, and every lane finishing its row by itself the pass over 1.08 GB took 229 us; now 172).
@@ -102,10 +82,13 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
     const int g = threadIdx.x >> 3, t = threadIdx.x & 7;
     const int r0 = blockIdx.x * rows_per_part, r1 = min(n, r0 + rows_per_part);
     const float* m4 = mu + static_cast<size_t>(u) * kMuStride;
-    float2 w[8];
+    float2 w[8];   // w[j] = channels j and 4 + j of the lane's first eight, w[4 + j] of its last eight: the chains of lane_dot16 in pairs
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        anchor_pairs(*reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h)), *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h + 4)), w + 4 * h);
+    for (int h = 0; h < 2; ++h) {
+        const float4 x = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h)), y = *reinterpret_cast<const float4*>(m4 + lane_channel(t, 8 * h + 4));
+        w[4 * h] = make_float2(x.x, y.x); w[4 * h + 1] = make_float2(x.y, y.y);
+        w[4 * h + 2] = make_float2(x.z, y.z); w[4 * h + 3] = make_float2(x.w, y.w);
+    }
     const float m = m4[kHeadDim];
     float* out = scores + static_cast<size_t>(u) * nmax;
 #pragma unroll 1
@@ -123,7 +106,20 @@ wide_score_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ n
         float ss[kWideDeep];
         double dot[kWideDeep];
 #pragma unroll
-        for (int k = 0; k < kWideDeep; ++k) lane_sumsq_dot_pairs(a[k], b[k], w, ss[k], dot[k]);
+        for (int k = 0; k < kWideDeep; ++k) {   // lane_sumsq and lane_dot16 in packed pairs
+            float x[16];
+            unpack_row(a[k], b[k], x);
+            float2 q = make_float2(0.f, 0.f), c0 = q, c1 = q;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) { const float2 v = make_float2(x[j], x[8 + j]); q = __ffma2_rn(v, v, q); }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                c0 = __ffma2_rn(make_float2(x[j], x[4 + j]), w[j], c0);
+                c1 = __ffma2_rn(make_float2(x[8 + j], x[12 + j]), w[4 + j], c1);
+            }
+            ss[k] = q.x + q.y;
+            dot[k] = (static_cast<double>(c0.x) + static_cast<double>(c0.y)) + (static_cast<double>(c1.x) + static_cast<double>(c1.y));
+        }
         const float r = sqrtf(group_sum_of4(ss, t));
         const float e = eviction_score(static_cast<float>(group_sum_of4(dot, t)), m, r, eps);
         const int i = base + (2 * (t & 1) + ((t >> 1) & 1)) * kWideGroups + g;
@@ -151,56 +147,13 @@ __device__ __forceinline__ void load_keys(const float* sc, int n, int scored, bo
         for (int i = tid; i < n; i += kSelThreads) keys[i] = i < scored ? order_key(__ldcg(&sc[i])) : 0xffffffffu;
     }
 }
-// Behind the selection, by 256 threads: tokens evicted in front of every word of the bitmap (n of them in all), and their list, ascending;
-// list may lie where the keys were.  Returns the first evicted token (E >= 1).
-__device__ __forceinline__ int list_evicted(int n, int tid, const Selector& s, int* before, int* list) {
-    const int nwords = (n + 31) >> 5;
-    const int per = (nwords + kSelThreads - 1) / kSelThreads, w0 = min(nwords, tid * per), w1 = min(nwords, w0 + per);
-    int cnt = 0;
-    for (int q = w0; q < w1; ++q) cnt += __popc(s.bitmap[q]);
-    int run = sel_exclusive_scan(cnt, tid, s.wtot);
-    for (int q = w0; q < w1; ++q) {
-        before[q] = run;
-        for (uint32_t wd = s.bitmap[q]; wd; wd &= wd - 1) list[run++] = 32 * q + __ffs(wd) - 1;
-    }
-    __syncthreads();
-    return list[0];
-}
-// The kept-index list (ascending) and the evicted rows' terms off the running sum, if one is kept.  table: [8][128] doubles.
-__device__ __forceinline__ void finish_unit(int u, int tid, const uint4* k_cache, const uint4* new_k, int len, int B, int N, float eps, int raw_anchor,
-                                            double* anchor_sum, int32_t* kept_idx, int32_t* mirror, int32_t* first_evicted,
-                                            unsigned long long* moved_rows, const Selector& s, int* before, int* gone, double* table) {
-    const int n = len + B, first = list_evicted(n, tid, s, before, gone);
-    double sum = 0.0;   // (requested in front of the rows)
-    if (anchor_sum && tid < kHeadDim) sum = __ldcg(&anchor_sum[static_cast<size_t>(u) * kHeadDim + tid]);
-    if (tid == 0) {
-        first_evicted[u] = first;
-        // block rows always move into the cache, cache rows only from the first evicted one on
-        atomicAdd(moved_rows, static_cast<unsigned long long>(N - min(len, first)));
-    }
-    int32_t* out = kept_idx + static_cast<size_t>(u) * N;
-    int32_t* out2 = mirror ? mirror + static_cast<size_t>(u) * N : nullptr;
-#pragma unroll 4
-    for (int i = tid; i < n; i += kSelThreads) {
-        const uint32_t wd = s.bitmap[i >> 5], bit = 1u << (i & 31);
-        if (!(wd & bit)) {
-            const int d = i - before[i >> 5] - __popc(wd & (bit - 1u));
-            out[d] = i;
-            if (out2) out2[d] = i;
-        }
-    }
-    if (!anchor_sum) return;   // (the staged path keeps no sum)
-    const double terms = block_sum_of_terms<kWideTermsDeep>(n - N, [&](int r) { return concat_row(k_cache, new_k, u, gone[r], len, B, N); },
-                                                            1.0f / eps, raw_anchor != 0, table, tid);
-    if (tid < kHeadDim) anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum - terms;
-}
-
 // Exact top-N of a unit (ties keep the older token), its kept-index list, and the evicted rows' terms off the running sum.
 // grid = U; dynamic shared memory: n keys (padded to four), two bitmaps.
 __global__ void __launch_bounds__(kSelThreads)
 wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ new_k, const float* __restrict__ scores,
                    int len, int B, int N, float eps, int raw_anchor, int nmax, int window, double* __restrict__ anchor_sum,
-                   int32_t* __restrict__ kept_idx, int32_t* __restrict__ first_evicted, unsigned long long* __restrict__ moved_rows) {
+                   int32_t* __restrict__ kept_idx, int32_t* __restrict__ first_evicted, unsigned long long* __restrict__ moved_rows,
+                   int32_t* status) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ __align__(128) SelectorScratch scratch;
     __shared__ __align__(16) double table[kTermWarps * kHeadDim];
@@ -212,8 +165,26 @@ wide_select_kernel(const uint4* __restrict__ k_cache, const uint4* __restrict__ 
     load_keys(scores + static_cast<size_t>(u) * nmax, n, n - window, (nmax & 3) == 0, keys, tid);
     __syncthreads();
     select_evicted(keys, n, n - N, tid, s);
-    finish_unit(u, tid, k_cache, new_k, len, B, N, eps, raw_anchor, anchor_sum, kept_idx, nullptr, first_evicted, moved_rows, s,
-                reinterpret_cast<int*>(s.eq), reinterpret_cast<int*>(keys), table);
+    int* before = reinterpret_cast<int*>(s.eq);
+    int* gone = reinterpret_cast<int*>(keys);   // (the keys are dead)
+    const int first = list_evicted(n, tid, s, before, gone, n - N, status);
+    double sum = 0.0;   // (requested in front of the rows)
+    if (anchor_sum && tid < kHeadDim) sum = __ldcg(&anchor_sum[static_cast<size_t>(u) * kHeadDim + tid]);
+    if (tid == 0) {
+        first_evicted[u] = first;
+        // block rows always move into the cache, cache rows only from the first evicted one on
+        atomicAdd(moved_rows, static_cast<unsigned long long>(N - min(len, first)));
+    }
+    int32_t* out = kept_idx + static_cast<size_t>(u) * N;
+#pragma unroll 4
+    for (int i = tid; i < n; i += kSelThreads) {
+        const uint32_t wd = bitmap[i >> 5], bit = 1u << (i & 31);
+        if (!(wd & bit)) out[i - before[i >> 5] - __popc(wd & (bit - 1u))] = i;
+    }
+    if (!anchor_sum) return;   // (the staged path keeps no sum)
+    const double terms = block_sum_of_terms<kWideTermsDeep>(n - N, [&](int r) { return concat_row(k_cache, new_k, u, gone[r], len, B, N); },
+                                                            1.0f / eps, raw_anchor != 0, table, tid);
+    if (tid < kHeadDim) anchor_sum[static_cast<size_t>(u) * kHeadDim + tid] = sum - terms;
 }
 
 // Step a4 in place by `segments` blocks per (unit, tensor): compact_kernel gives a tensor of a unit one block, which for fewer
