@@ -99,7 +99,8 @@ enum {
 enum {
     KEYDIFF_PATH_AUTO = 0,    /* one fused launch, or four (reported as KEYDIFF_PATH_STAGED) where a unit
                                  does not fit it or four are faster; many long units that evict a single
-                                 row take four in that step */
+                                 row take four in that step, and with slot reuse more long units than the
+                                 device has SMs may take two (reported as KEYDIFF_PATH_FUSED) */
     KEYDIFF_PATH_STAGED = 1,  /* four launches: anchor partials, scores, select, compaction; nothing but the
                                  caches is carried from step to step */
     KEYDIFF_PATH_FUSED = 2    /* one launch, one thread block or one cluster of them per unit; create fails
@@ -284,14 +285,17 @@ KEYDIFF_API int keydiff_set_positions(keydiff_ctx* ctx, const int32_t* pos_devic
 KEYDIFF_API int keydiff_get_moved_rows(const keydiff_ctx* ctx, const unsigned long long** counter);
 
 /* Launch facts of the chosen path, for benchmarks: path actually used (KEYDIFF_PATH_*), kernels launched per
- * evicting step, cluster size (1 where no cluster is used).  Not counted: with path STAGED reported for KEYDIFF_PATH_AUTO,
- * and with slot reuse in clusters or with several blocks per unit, a step that has to rebuild the running anchor sum (keydiff_set_incremental)
- * launches up to two more; and with KEYDIFF_PATH_AUTO a context of many long units in token order, whose steps are one launch,
- * makes four in a step that evicts a single row. */
+ * evicting step of max_block rows with the keydiff_set_incremental setting as it is, cluster size (1 where no cluster is used).  A step
+ * may differ from that.  One that has to rebuild the running anchor sum launches up to two more with path STAGED reported for
+ * KEYDIFF_PATH_AUTO, and with slot reuse in clusters or with several blocks per unit; or it is one launch of a block per unit where that can
+ * serve the units (about 4500 rows, or six units per SM and more).  There a step of fewer rows may take several blocks per unit, in two
+ * launches, although one of max_block rows does not.  And with KEYDIFF_PATH_AUTO a context of many long units in token order, whose
+ * steps are one launch, makes four in a step that evicts a single row. */
 KEYDIFF_API int keydiff_get_launch_info(const keydiff_ctx* ctx, int32_t* path, int32_t* launches_per_step,
                             int32_t* cluster_size);
 
-/* Name of the kernel, or of the group of four, that serves an evicting step; never NULL ("" for a NULL ctx). */
+/* Name of the kernel, or of the group of four, that serves an evicting step as keydiff_get_launch_info describes it; never NULL ("" for a
+ * NULL ctx).  Where two kernels serve it (several blocks per unit), the one that reads the keys. */
 KEYDIFF_API const char* keydiff_get_kernel_name(const keydiff_ctx* ctx);
 
 /*

@@ -598,8 +598,11 @@ bool parts_are_faster(const keydiff_ctx* c, int B) {
     return within(100, large ? 135 : 124) || within(200, 233) || within(300, 311);
 }
 
-// Whether the facts reported are those of several blocks per unit: a step of max_block rows.
-bool parts_named(const keydiff_ctx* c) { return c->parts && (!c->unit_blocks || parts_are_faster(c, c->cfg.max_block)); }
+// The facts reported are those of a step of max_block rows as the context stands: on the running sum, or without it for good
+// (keydiff_set_incremental), which a block per unit serves where it can.
+bool parts_named(const keydiff_ctx* c) {
+    return c->parts && (!c->unit_blocks || (c->incremental && parts_are_faster(c, c->cfg.max_block)));
+}
 
 // A block per unit rebuilds the sum by itself where that is needed, and goes on from the same sum.
 bool parts_serve(const keydiff_ctx* c, int B) { return c->parts && (!c->unit_blocks || (sum_valid(c) && parts_are_faster(c, B))); }

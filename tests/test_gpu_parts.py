@@ -48,6 +48,16 @@ def test_which_kernel_serves(U, N, B, kernel):
     kd.close()
 
 
+@pytest.mark.parametrize("U,N,B,carried,rebuilt", [(150, 2048, 64, "parts_kernel", "unit_evict_kernel"), (1000, 8192, 64, "parts_kernel", "unit_evict_kernel"),
+                                                    (150, 8192, 64, "parts_kernel", "parts_kernel"), (177, 2300, 512, "unit_evict_kernel", "unit_evict_kernel")])
+def test_the_facts_reported_are_those_of_a_step_as_the_context_stands(U, N, B, carried, rebuilt):
+    kd = KeyDiff(1, 1, U, 128, N, B, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
+    for on, kernel in ((True, carried), (False, rebuilt), (True, carried)):
+        kd.set_incremental(on)
+        assert kd.kernel_name() == kernel and kd.launch_info()["launches_per_step"] == (2 if kernel == "parts_kernel" else 1)
+    kd.close()
+
+
 @pytest.mark.parametrize("N", [2000, 4600])
 def test_captured_steps_and_the_host_entry_give_the_same(N):
     U, B = 150, 64
