@@ -31,6 +31,9 @@ __device__ __forceinline__ bool bad_row(int32_t* status) {   // status may be nu
 // positions, the cluster kernels before their last barrier; a successor waits for all of it): blocks that move in earlier and wait
 // cost the kernels that fill the SMs' shared memory 0.7-1.3 % of a step, and the four launches of a step on 256 units of 16512
 // rows 1138 instead of 902 us.
+// One pair is an exception to both: wide_anchor_kernel lets parts_kernel in at its start, and that one requests keys from k_cache and new_k before it
+// waits.  This is right only because the trigger stands behind wide_anchor_kernel's own wait (all that wrote the two tensors is complete
+// by then) and wide_anchor_kernel itself writes neither.  No other kernel may be put between the two or take the first one's place.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

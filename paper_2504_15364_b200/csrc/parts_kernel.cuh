@@ -52,8 +52,8 @@ __device__ __forceinline__ void score_rows(const UnitParams& p, const float* mu,
         }
     };
     const int first = r0 + 16 * warp;
-    load(first);
-    grid_dependency_wait();   // the anchors (the kernel that forms them lets this one in when everything before it is complete)
+    load(first);              // (in front of the wait: the kernel that forms the anchors lets this one in when everything before it is complete)
+    grid_dependency_wait();   // the anchors
     mu += static_cast<size_t>(u) * kMuStride;
     float2 w[8];
     load_anchor(mu, t, w);

@@ -35,7 +35,9 @@ wide_anchor_kernel(const uint4* __restrict__ new_k, int B, int n, float eps, int
     __shared__ __align__(16) double table[kTermWarps * kHeadDim];
     __shared__ float mu_sh[kHeadDim];
     grid_dependency_wait();
-    if (let_in) grid_dependency_trigger();   // parts_kernel, which requests keys before it waits for the anchors
+    // parts_kernel requests keys and block rows before it waits for the anchors: let in behind the wait above, never in front of it, and nothing here
+    // writes either tensor (common.cuh)
+    if (let_in) grid_dependency_trigger();
     const int u = blockIdx.x, tid = threadIdx.x;
     const uint4* blk = new_k + static_cast<size_t>(u) * B * kRowVec;
     if (move_sync && tid < 2 * kMaxSegments) move_sync[1 + u * 2 * kMaxSegments + tid] = 0u;

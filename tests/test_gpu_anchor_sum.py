@@ -52,10 +52,13 @@ CHILD = textwrap.dedent("""
 
 
 # steps of the cluster kernel and single rows through the four launches (what came in a block goes by itself and the other way round:
-# N is three and a half turns); the same on the raw anchor; the four launches alone; one block per unit; slot reuse, one block and clusters
+# N is three and a half turns); the same on the raw anchor; the four launches alone; one block per unit; slot reuse, one block and clusters;
+# several blocks per unit, their steps in turn with a block per unit's (which rebuilds the sum every 1024 steps, and takes the large blocks)
 @pytest.mark.parametrize("args,cluster", [((185, 2100, 2400, 0, 0, 500) + (1,) * 100, 0), ((300, 2048, 2072, 0, 1, 33, 1, 1, 2), 0),
                                           ((3, 1500, 1656, 0, 0, 97, 1, 40), 1), ((90, 240, 276, 0, 0, 16, 7), 0),
-                                          ((8, 500, 606, 1, 0, 100, 1), 0), ((8, 4000, 4128, 1, 0, 128, 1), 0)])
+                                          ((8, 500, 606, 1, 0, 100, 1), 0), ((8, 4000, 4128, 1, 0, 128, 1), 0),
+                                          ((150, 4600, 4692, 1, 0, 64, 5), 0), ((150, 2000, 2100, 1, 0, 100) + (1,) * 600, 0),
+                                          ((150, 2400, 2756, 1, 1, 600, 64, 20, 5), 0)])
 def test_the_sum_is_unchanged_when_the_rows_are(args, cluster):
     build.build_library()
     build.build_library(debug_checks=True)

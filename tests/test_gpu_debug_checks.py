@@ -19,10 +19,11 @@ CHILD = textwrap.dedent("""
     binding.LIB_PATH = build.DEBUG_LIB if sys.argv[1] == "debug" else build.LIB
     from paper_2504_15364_b200 import KeyDiff
     out = []
-    for comp, path, N, B in [(0, 2, 1536, 128), (1, 2, 1536, 128), (0, 1, 700, 33), (1, 1, 700, 33), (0, 2, 9000, 300)]:
-        wl = synth.Workload("t", 1, 2, 3, 128, N, B, "outlier", N + 4 * B, 77)
+    for comp, path, N, B, heads in [(0, 2, 1536, 128, 3), (1, 2, 1536, 128, 3), (0, 1, 700, 33, 3), (1, 1, 700, 33, 3), (0, 2, 9000, 300, 3),
+                                    (1, 0, 2000, 64, 75), (1, 0, 4600, 33, 75), (0, 0, 10600, 50, 30), (1, 0, 300, 40, 75), (0, 0, 300, 40, 75)]:
+        wl = synth.Workload("t", 1, 2, heads, 128, N, B, "outlier", N + 4 * B, 77)
         k_cache, v_cache, stream = synth.prefilled_cache(wl, "cuda")
-        kd = KeyDiff(1, 2, 3, 128, N, B, path=path, compaction=comp, recent_window=40)
+        kd = KeyDiff(1, 2, heads, 128, N, B, path=path, compaction=comp, recent_window=40)
         kd.set_len(N)
         for _ in range(4):
             kd.evict(k_cache, v_cache, *stream.next_block())

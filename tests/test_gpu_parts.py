@@ -14,6 +14,8 @@ pytestmark = pytest.mark.gpu
     (177, 2047, 2000, (130, 130, 7), 400, 0, "clusters"),         # the first step also fills empty slots; single keys, window beyond the block
     (160, 2304, 2304, (1, 256, 1, 255), 20, 1, "drift"),
     (450, 1999, 1999, (3, 3), 0, 0, "offset"),
+    (150, 2001, 2001, (40, 9, 40), 1500, 1, "clusters"),          # windows far beyond a block, positions out of order
+    (300, 4601, 4601, (33, 33), 4600, 0, "drift"),
     (150, 4600, 4600, (33, 33, 1), 0, 0, "outlier"),              # the first sum comes from launches of its own
     (149, 10200, 10200, (64, 64), 0, 0, "drift"),                 # two blocks per SM, though three would fit
     (149, 13000, 13000, (64, 64), 0, 0, "outlier"),               # two fit
@@ -21,6 +23,47 @@ pytestmark = pytest.mark.gpu
     (150, 3900, 3900, (700, 5, 700), 900, 0, "outlier")])
 def test_steps_match_the_oracle(U, N, length, blocks, window, raw, model):
     check_steps(U, N, max(blocks), length, True, model=model, kernel="parts_kernel", blocks=blocks, recent_window=window, anchor_mode=raw)
+
+
+def steps_of(path, k0, v0, blocks, window, incremental=True, reset_at=None):
+    """What the steps leave, from a copy of a full cache; with reset_at the step of that number is the first of a new sequence over the same rows."""
+    U, N = k0.shape[0], k0.shape[1]
+    k, v = k0.clone(), v0.clone()
+    kd = KeyDiff(1, 1, U, 128, N, max(b[0].shape[-2] for b in blocks), path=path, recent_window=window, compaction=binding.KEYDIFF_COMPACT_SLOT_REUSE)
+    kd.set_incremental(incremental)
+    kd.set_len(N)
+    scores = []
+    for i, b in enumerate(blocks):
+        if i == reset_at:
+            kd.reset()
+            kd.set_len(N)
+        kd.evict(k, v, *b)
+        scores.append(kd.scratch()["scores"].clone())
+    torch.cuda.synchronize()
+    assert int(kd.scratch()["status"].item()) == 0
+    out = k, v, kd.positions()[0].clone(), kd.scratch()["kept_idx"].clone(), torch.stack(scores)
+    name = kd.kernel_name()
+    kd.close()
+    return name, out
+
+
+@pytest.mark.parametrize("U,N,B,window,incremental,reset_at", [(150, 2000, 64, 0, True, None), (450, 2047, 100, 600, True, None), (150, 2000, 64, 300, True, 2),
+                                                               (150, 2000, 64, 0, False, None), (150, 4600, 33, 0, True, None), (300, 4500, 64, 1000, True, 2),
+                                                               (150, 4600, 33, 0, False, 1)])
+def test_the_kernels_that_serve_these_shapes_with_the_fused_path_agree(U, N, B, window, incremental, reset_at):
+    wl = synth.Workload("t", 1, 1, U, 128, N, B, "drift", N + 5 * B, 93)
+    k0, v0, stream = synth.prefilled_cache(wl, "cuda")
+    blocks = [stream.next_block(b) for b in (B, B, 1, B)]
+    name, out = steps_of(binding.KEYDIFF_PATH_AUTO, k0, v0, blocks, window, incremental, reset_at)
+    old, ref = steps_of(binding.KEYDIFF_PATH_FUSED, k0, v0, blocks, window, incremental, reset_at)
+    assert name == ("parts_kernel" if incremental or N > 4400 else "unit_evict_kernel") and old == ("unit_evict_kernel" if N < 4400 else "slot_evict_kernel")
+    if old == "unit_evict_kernel":   # the same additions in the same order
+        assert all(torch.equal(a, b) for a, b in zip(out, ref))
+        return
+    # A unit's cluster adds the same terms in another order (block rows and evicted ones together): sums in double, an anchor that may round
+    # the other way in fp32, 2^-24 of it, and with it the scores: 128 products, 2^-24 each at most of |mu| |k|.
+    assert all(torch.equal(a, b) for a, b in zip(out[:4], ref[:4]))
+    assert float((out[4] - ref[4]).abs().max()) <= 2.0 ** -24 * 128
 
 
 @pytest.mark.parametrize("U,N,blocks,window", [(160, 2500, (600, 1, 600, 64, 512, 513), 0), (640, 1950, (384, 16, 384, 1), 500)])

@@ -42,17 +42,18 @@ def test_a_bounded_wait_that_runs_out_reports_timeout_and_the_context_stays_usab
 
 
 @pytest.mark.parametrize("compaction", [binding.KEYDIFF_COMPACT_ORDERED, binding.KEYDIFF_COMPACT_SLOT_REUSE])
-def test_allocation_failure_in_create_releases_everything(compaction):
+@pytest.mark.parametrize("units,N", [((2, 1, 4), 1024), ((1, 1, 150), 2048), ((1, 1, 190), 2048)])   # 150: several blocks per unit, 190: launches for single rows
+def test_allocation_failure_in_create_releases_everything(compaction, units, N):
     torch.cuda.synchronize()
     args = dict(path=binding.KEYDIFF_PATH_AUTO, compaction=compaction)
-    KeyDiff(2, 1, 4, 128, 1024, 64, **args).close()          # warm: module loading, attributes
+    KeyDiff(*units, 128, N, 64, **args).close()          # warm: module loading, attributes
     torch.cuda.synchronize()
     free0 = torch.cuda.mem_get_info()[0]
     failures = 0
     for nth in range(1, 16):
         binding.debug_fail_alloc(nth)
         try:
-            kd = KeyDiff(2, 1, 4, 128, 1024, 64, **args)
+            kd = KeyDiff(*units, 128, N, 64, **args)
         except KeyDiffError as e:
             assert e.code == binding.KEYDIFF_ERR_ALLOC
             failures += 1
@@ -62,7 +63,7 @@ def test_allocation_failure_in_create_releases_everything(compaction):
     assert failures >= 10, failures          # every allocation of keydiff_create was made to fail once
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] >= free0 - (2 << 20), "a failed keydiff_create leaked device memory"
-    kd = KeyDiff(2, 1, 4, 128, 1024, 64, **args)            # and the library still works
+    kd = KeyDiff(*units, 128, N, 64, **args)            # and the library still works
     kd.close()
 
 
