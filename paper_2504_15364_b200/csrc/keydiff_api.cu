@@ -348,8 +348,8 @@ int launch_slot_stream(keydiff_ctx* c, uint4* kc, uint4* vc, const uint4* nk, co
     // Start-up stagger: clusters launched together stream together and then select together, leaving HBM
     // idle in between.  When every cluster serves at least three units, starting cluster c a little later
     // than cluster c-1 (about half a unit's duration over all of them) spreads the phases; with fewer
-    // units per cluster the delay would only postpone the end (sweep on a B200: 896 units of 4352 rows
-    // gain 12 %, 256 units of 8320 rows lose 3 %).
+    // units per cluster the delay would only postpone the end (sweep on a B200, by this kernel whichever serves
+    // the shape now: 896 units of 4352 rows gain 12 %, 256 units of 8320 rows lose 3 %).
     p.stagger_ns = 0;
     p.late_ns = 0;
     {
@@ -388,7 +388,8 @@ UnitKernel unit_instance(const keydiff_ctx* c) {   // unit_depth 0, and the orde
 //   slot reuse       nothing but the block rows is read twice: 400 x 2112 54 / 69, 1000 x 4160 226 / 237, 800 x 1764 131 / 160.
 //                    148 units or fewer: up to 1100 rows, 100 x 1064 17.8 / 18.5, 100 x 2112 25 / 23; a few units up to 600
 //                    rows, 8 x 564 14 / 15, 8 x 1064 18 / 15.  Beyond 4500 rows only with many rounds
-//                    of units: 600 x 8224 268 / 263, 1000 x 8224 377 / 388, 4096 x 8224 1381 / 1460.
+//                    of units: 600 x 8224 268 / 263, 1000 x 8224 377 / 388, 4096 x 8224 1381 / 1460.  (These are the two kernels alone;
+//                    where several blocks per unit are faster than either, parts_are_faster says so: 1000 x 4160, 600 and 1000 x 8224.)
 // The ring (rows through shared memory by the copy engine) needs shared memory that short units' blocks put to better use: 800 x
 // 1764 142 with it, 131 without; with at most two blocks per SM, or long units, it is what keeps HBM busy: 224 x 2176 44 / 45,
 // 200 x 4160 59 / 64, 1000 x 8224 376 / 437, 2000 x 8224 697 / 826.

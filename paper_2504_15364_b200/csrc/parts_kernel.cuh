@@ -3,10 +3,10 @@
 // formed by wide_anchor_kernel from the running sum.  No block waits for another one.
 //
 // A unit's rows are read once, and a unit is no longer tied to one block: the units need not fill the SMs in whole rounds, and of all
-// selections only the last ones are not hidden behind the reading of keys.  What bounds it: HBM (1000 x 8256 rows 362 us a step, 5.8 TB/s),
+// selections only the last ones are not hidden behind the reading of keys.  What bounds it: HBM (1000 x 8256 rows 365 us a step, 5.8 TB/s),
 // and at the ends about 5 us for the anchors and a chain of 13 us (units of 2000 rows) to 19 us (8000) for the last unit: keys 2, selection 6,
 // lists 3, evicted rows 4, placement 3.  Against a block per unit, or per unit and round, us a step: 300 x 8256 rows 172 -> 125, 180 x 8256 119 -> 84,
-// 512 x 4160 140 -> 115, 896 x 4352 246 -> 220, 1000 x 8256 385 -> 362, 160 x 16448 182 -> 145.
+// 512 x 4160 140 -> 115, 896 x 4352 246 -> 220 (256 a step: 263 -> 240), 1000 x 8256 388 -> 365, 160 x 16448 182 -> 145.
 #pragma once
 #include "unit_kernel.cuh"
 #include "wide_kernels.cuh"

@@ -5,10 +5,11 @@
 // chip and fill an SM with one block, which for a unit of a few hundred rows is latency from end to end.)
 //
 // What bounds it: three blocks per SM (80 registers, by launch bounds; at 64 registers and four blocks most shapes lose 3-10 %)
-// work through a chain of about 14 us for a unit of 300 rows: 1344 x 316 rows 188 -> 97 us a step, with slot reuse 165 -> 81.
-// Long units: HBM, with slot reuse (1000 x 8224 rows 376 us, 335 at the copy rate; 2000 x 8224 697, 670).
+// work through a chain of about 14 us for a unit of 300 rows: 1344 x 316 rows, 16 a step, in clusters of one
+// and here, 169 -> 102 us in token order, 155 -> 53 with slot reuse.
+// Long units: HBM, with slot reuse (2000 x 8224 rows, 32 a step, 690-730 us, 683 at the copy rate).
 // The ring's 64 KB leave room for two blocks per SM: on 224 x 2176 rows the 224 blocks are all there at once, and the step is
-// one chain (143 MB of traffic in 44 us, issue slots 43 % busy).
+// one chain (143 MB of traffic in 46 us, issue slots 43 % busy).
 #pragma once
 #include "evicted_list.cuh"
 #include "row_terms.cuh"
@@ -80,7 +81,7 @@ __device__ __forceinline__ void place_block_rows(const UnitParams& p, int u, int
         if (!evicted(i) && KD_ROW_OK(at, p.max_block, p.status)) blk_of[at] = j;
     }
     // kept cache rows keep their slot.  Four entries at a time where they can be (an evicted row's entry is written again below, behind a barrier):
-    // 1344 x 316 rows 51.6 -> 49.7 us a step, 4096 x 8224 1390 -> 1377, 1000 x 8256 385 -> 381
+    // 1344 x 316 rows 51.6 -> 49.7 us a step
     if (((N | len) & 3) == 0 && !mirror) {
         int4* kept4 = reinterpret_cast<int4*>(kept);
 #pragma unroll 4

@@ -10,7 +10,7 @@
 // The running sum cannot drift: a row's terms are the fixed bit pattern that the other kernels add and take out as well
 // (row_terms.cuh), added and subtracted in double.
 //
-// What bounds it: HBM.  256 units of 16512 keys, 5.4 GB of traffic a step: 891 us; in the staged kernels 1280 us (anchor and
+// What bounds it: HBM.  256 units of 16512 keys, 5.4 GB of traffic a step: 886 us; in the staged kernels 1280 us (anchor and
 // score pass 308 + 229, selection 66, compaction 684).  The score pass takes 172 us (6.3 TB/s), the selection 25, the
 // compaction 679 (6.3 TB/s, and the last units' keys from L2).
 #pragma once

@@ -1,5 +1,5 @@
-"""Slot reuse with several blocks per unit (csrc/parts_kernel.cuh): more units than SMs whose last round would be far from full, against the
-oracle; ragged parts, both variants, transition steps, blocks of one row, either way to the first sum, host entry and capture."""
+"""Slot reuse with several blocks per unit (csrc/parts_kernel.cuh) against the oracle: ragged parts, both variants, transition steps, blocks of one row,
+either way to the first sum, host entry and capture; which kernel serves which shape and step, and what the others give for the same steps."""
 import pytest
 import torch
 

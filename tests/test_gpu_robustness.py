@@ -42,8 +42,10 @@ def test_a_bounded_wait_that_runs_out_reports_timeout_and_the_context_stays_usab
 
 
 @pytest.mark.parametrize("compaction", [binding.KEYDIFF_COMPACT_ORDERED, binding.KEYDIFF_COMPACT_SLOT_REUSE])
-@pytest.mark.parametrize("units,N", [((2, 1, 4), 1024), ((1, 1, 150), 2048), ((1, 1, 190), 2048)])   # 150: several blocks per unit, 190: launches for single rows
-def test_allocation_failure_in_create_releases_everything(compaction, units, N):
+# 150 units with slot reuse: several blocks per unit; 190 in token order: launches for single rows, with slot reuse: a block per unit, which needs one
+# buffer beside the eight of every such context
+@pytest.mark.parametrize("units,N,least", [((2, 1, 4), 1024, 10), ((1, 1, 150), 2048, 10), ((1, 1, 190), 2048, 9)])
+def test_allocation_failure_in_create_releases_everything(compaction, units, N, least):
     torch.cuda.synchronize()
     args = dict(path=binding.KEYDIFF_PATH_AUTO, compaction=compaction)
     KeyDiff(*units, 128, N, 64, **args).close()          # warm: module loading, attributes
@@ -60,7 +62,7 @@ def test_allocation_failure_in_create_releases_everything(compaction, units, N):
             continue
         kd.close()        # nth is past the last allocation of create: the hook was disarmed by create's return
         break
-    assert failures >= 10, failures          # every allocation of keydiff_create was made to fail once
+    assert failures >= least, failures       # every allocation of keydiff_create was made to fail once
     torch.cuda.synchronize()
     assert torch.cuda.mem_get_info()[0] >= free0 - (2 << 20), "a failed keydiff_create leaked device memory"
     kd = KeyDiff(*units, 128, N, 64, **args)            # and the library still works
